@@ -337,6 +337,10 @@ def _transform(n):
     return ((C @ IZ) / C[:, :1]).cuda()
 
 
+def _inverse(M):
+    return torch.from_numpy(np.linalg.inv(M.cpu().numpy())).cuda()
+
+
 def _m3(T, X):
     return (T @ X.reshape(X.shape[0], -1)).reshape(X.shape)
 
@@ -346,7 +350,7 @@ def _op(A, B, X):
     Z = torch.bmm(_m3(M, A), _m3(M, X))
     if B is not None:
         Z = torch.bmm(Z, _m3(M, B))
-    return _m3(torch.linalg.inv(M), Z)
+    return _m3(_inverse(M), Z)
 
 
 class _Operator:
@@ -354,7 +358,7 @@ class _Operator:
 
     def __init__(self, A, B):
         self.M = _transform(A.shape[0])
-        self.Mi = torch.linalg.inv(self.M)
+        self.Mi = _inverse(self.M)
         self.A = _m3(self.M, A.double())
         self.B = None if B is None else _m3(self.M, B.double())
 
