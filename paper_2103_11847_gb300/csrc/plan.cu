@@ -143,8 +143,9 @@ int cprod_epi(tc_plan* p, const float* X, float* Y, const Epi& ep, cudaStream_t 
   mid.skip = ep.skip;
   if (fused(p)) {
     if (!p->two_sided)
-      return launch_slice_gemm(p->Ah, X, Y, n1, s, n2, n3, p->hM, p->hMinv, ep, st);
-    TC_TRY(launch_slice_gemm(p->Ah, X, p->tmp1, n1, s, n2, n3, p->hM, nullptr, mid, st));
+      return launch_slice_gemm(p->AhT, X, Y, n1, s, n2, n3, p->hM, p->hMinv, ep, st);
+    TC_TRY(launch_slice_gemm(p->AhT, X, p->tmp1, n1, s, n2, n3, p->hM, nullptr, mid, st, true,
+                             ep.red.out != nullptr));
     return launch_slice_gemm(p->tmp1, p->Bh, Y, n1, s, s, n3, nullptr, p->hMinv, ep, st);
   }
   if (lowp(p)) {  // transform to the GEMM input type, tcgen05 slice GEMMs, transform back
@@ -174,7 +175,8 @@ int cprod_epi(tc_plan* p, const float* X, float* Y, const Epi& ep, cudaStream_t 
                : launch_mode3(p->tmp2, Y, p->dMinv, n3, (size_t)n1 * s, ep, st);
   }
   TC_TRY(launch_mode3(X, p->tmp1, p->dM, n3, (size_t)n2 * s, mid, st));
-  TC_TRY(launch_slice_gemm(p->Ah, p->tmp1, p->tmp2, n1, s, n2, n3, nullptr, nullptr, mid, st));
+  TC_TRY(launch_slice_gemm(p->AhT, p->tmp1, p->tmp2, n1, s, n2, n3, nullptr, nullptr, mid, st,
+                           p->two_sided));
   const float* src = p->tmp2;
   if (p->two_sided) {
     TC_TRY(launch_slice_gemm(p->tmp2, p->Bh, p->tmp1, n1, s, s, n3, nullptr, nullptr, mid, st));
@@ -215,7 +217,8 @@ int cprod_td(tc_plan* p, const float* Xt, float* Yt, const Epi& ep, cudaStream_t
     TC_TRY(launch_umma(*p->umf, p->tmp2, err, ep.skip, st));
     if (p->two_sided) TC_TRY(right_factor(p, *p->umf2, (size_t)n1 * s * n3, err, ep.skip, st));
   } else {
-    TC_TRY(launch_slice_gemm(p->Ah, Xt, p->tmp2, n1, s, n2, n3, nullptr, nullptr, mid, st));
+    TC_TRY(launch_slice_gemm(p->AhT, Xt, p->tmp2, n1, s, n2, n3, nullptr, nullptr, mid, st,
+                             p->two_sided));
     if (p->two_sided) {
       TC_TRY(launch_slice_gemm(p->tmp2, p->Bh, p->tmp1, n1, s, s, n3, nullptr, nullptr, mid, st));
       src = p->tmp1;
@@ -280,7 +283,8 @@ int adjoint_td(tc_plan* p, const float* Yt, float* Xt, const Epi& ep, cudaStream
     TC_TRY(launch_umma(*p->uma, p->tmp2, err, ep.skip, st));
     if (p->two_sided) TC_TRY(right_factor(p, *p->uma2, (size_t)n2 * s * n3, err, ep.skip, st));
   } else {
-    TC_TRY(launch_slice_gemm(p->AhT, Yt, p->tmp2, n2, s, n1, n3, nullptr, nullptr, mid, st));
+    TC_TRY(launch_slice_gemm(p->Ah, Yt, p->tmp2, n2, s, n1, n3, nullptr, nullptr, mid, st,
+                             p->two_sided));
     if (p->two_sided) {
       TC_TRY(launch_slice_gemm(p->tmp2, p->BhT, p->tmp1, n2, s, s, n3, nullptr, nullptr, mid, st));
       src = p->tmp1;
@@ -303,11 +307,12 @@ int adjoint_epi(tc_plan* p, const float* Y, float* X, const Epi& ep, cudaStream_
   mid.skip = ep.skip;
   if (fused(p)) {
     if (!p->two_sided)
-      return launch_slice_gemm(p->AhT, Y, X, n2, s, n1, n3, p->hMinvT, p->hMT, ep, st);
+      return launch_slice_gemm(p->Ah, Y, X, n2, s, n1, n3, p->hMinvT, p->hMT, ep, st);
     if (cprod2_fits(s))
       return launch_cprod2(p->Ah, Y, p->BhT, X, n2, n1, s, n3, p->hMinvT, p->hMT, ep,
                            LsqrStep{}, st);
-    TC_TRY(launch_slice_gemm(p->AhT, Y, p->tmp1, n2, s, n1, n3, p->hMinvT, nullptr, mid, st));
+    TC_TRY(launch_slice_gemm(p->Ah, Y, p->tmp1, n2, s, n1, n3, p->hMinvT, nullptr, mid, st, true,
+                             ep.red.out != nullptr));
     return launch_slice_gemm(p->tmp1, p->BhT, X, n2, s, s, n3, nullptr, p->hMT, ep, st);
   }
   if (lowp(p)) {
@@ -338,7 +343,8 @@ int adjoint_epi(tc_plan* p, const float* Y, float* X, const Epi& ep, cudaStream_
                : launch_mode3(p->tmp2, X, p->dMT, n3, (size_t)n2 * s, ep, st);
   }
   TC_TRY(launch_mode3(Y, p->tmp1, p->dMinvT, n3, (size_t)n1 * s, mid, st));
-  TC_TRY(launch_slice_gemm(p->AhT, p->tmp1, p->tmp2, n2, s, n1, n3, nullptr, nullptr, mid, st));
+  TC_TRY(launch_slice_gemm(p->Ah, p->tmp1, p->tmp2, n2, s, n1, n3, nullptr, nullptr, mid, st,
+                           p->two_sided));
   const float* src = p->tmp2;
   if (p->two_sided) {
     TC_TRY(launch_slice_gemm(p->tmp2, p->BhT, p->tmp1, n2, s, s, n3, nullptr, nullptr, mid, st));
@@ -609,7 +615,7 @@ extern "C" int tc_slice_gemm(tc_plan* p, const void* Xh, float* Yh, int adjoint,
   const int M = adjoint ? p->n2 : p->n1, K = adjoint ? p->n1 : p->n2;
   if (!lowp(p)) {
     Epi none;
-    return launch_slice_gemm(adjoint ? p->AhT : p->Ah, static_cast<const float*>(Xh), Yh, M,
+    return launch_slice_gemm(adjoint ? p->Ah : p->AhT, static_cast<const float*>(Xh), Yh, M,
                              p->s, K, p->n3, nullptr, nullptr, none, st);
   }
   const void* bop = Xh;

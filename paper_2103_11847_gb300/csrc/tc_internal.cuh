@@ -173,12 +173,16 @@ void tc_set_message(const char* msg);
 
 // ---------------------------------------------------------- kernel drivers --
 // gemm.cu: C_k = A_k * (pro-transformed B)_k for nslices slices, epilogue.
-// A: M x K per slice (row-major), B: K x N, C/prev: M x N; slice strides are
-// the dense sizes. pro/epi: n3 x n3 row-major (host arrays, by value), used
-// only when the CTA owns all n3 <= TC_MAX_FUSED slices.
-int launch_slice_gemm(const float* A, const float* B, float* C, int M, int N, int K,
+// At: the left factor K-major (K x M per slice, row-major: A_k^T), B: K x N,
+// C/prev: M x N; slice strides are the dense sizes. pro/epi: n3 x n3 row-major
+// (host arrays, by value), used only when the CTA owns all n3 <= TC_MAX_FUSED
+// slices. trans: C is stored N x M a slice (the K-major left factor of a
+// second product; no prev and no reduction). solve: a solver's product, whose
+// order of additions does not follow the tile chosen (implied by ep.red).
+int gemm_init();
+int launch_slice_gemm(const float* At, const float* B, float* C, int M, int N, int K,
                       int nslices, const float* pro, const float* epi, const Epi& ep,
-                      cudaStream_t st);
+                      cudaStream_t st, bool trans = false, bool solve = false);
 // gemm2.cu: the whole two-sided fused product Y = epi[ A_k (pro X)_k B_k ]
 // in one launch of thread-block clusters, for N = s <= 256 (cprod2_fits).
 // At: the left factor K-major (K x M per slice: A_k^T), X: K x N, B: N x N,
