@@ -275,7 +275,6 @@ __device__ __forceinline__ void reduce_blocks(const float (&v)[2], const Red& re
   constexpr int NW = 4 * V;             // (virtual) warps a block
   constexpr int B = T::BM / 64;         // blocks a CTA
   __shared__ float sh_f[B * NW];
-  __shared__ double sh_d[NW];
   __shared__ int sh_last;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   float s = v[0];
@@ -306,26 +305,7 @@ __device__ __forceinline__ void reduce_blocks(const float (&v)[2], const Red& re
     }
   }
   __syncthreads();
-  if (!sh_last) return;
-  if (tid < 128) {
-#pragma unroll
-    for (int q = 0; q < V; ++q) {
-      double acc = 0.0;
-      for (unsigned i = tid + 128 * q; i < nblk; i += 128 * V) acc += __ldcg(red.partials + i);
-      acc = warp_sum(acc);
-      if (lane == 0) sh_d[4 * q + w] = acc;
-    }
-  }
-  __syncthreads();
-  if (tid < 32) {
-    double t = lane < NW ? sh_d[lane] : 0.0;
-    t = warp_sum(t);
-    if (tid == 0) {
-      if (red.status && !isfinite(t)) *red.status = TC_ENONFINITE;
-      *red.out = red.sqrt_out ? sqrt(t) : t;
-      *red.ticket = 0u;
-    }
-  }
+  if (sh_last) sum_partials<V>(red, nblk);
 }
 
 __device__ __forceinline__ Out make_out(float* C, const Epi& ep, bool trans, int M, int N, float ca,
@@ -587,15 +567,14 @@ using TileM = ftile::Tile<NS, 64, 64, 16, 4, 3, true>;
 //   n = 320 [2.5]: 14.5 / 30.8 / 14.4    384 [4.4]: 20.3 / 34.9 / 16.5
 //   n = 512 [10.4]: 40.3 / 45.2 / 27.9   768 [35]: 105 / 65.6 / 65.6
 //   n = 1024 [83]: 248 / 156 / 140
-// Up to 20 64 x 64 tiles the launch is a latency: small tiles, K split until
-// the grid covers the SMs. Above, the SMs that take the most tiles set the
+// Up to 20 64 x 64 tiles the launch is a latency: small tiles, K split while
+// the grid does not cover the SMs and each rank keeps two K blocks. Above, the SMs that take the most tiles set the
 // time: ceil(tiles KS / SMs) / KS, smallest over KS = 1, 2, 4, 8 (each rank
 // keeps at least two K blocks). Ties: four ranks where a whole tile each leaves
 // SMs idle (more warps a SM), no split where it does not (no exchange).
 // A solver's products (ep.red, or `solve` for the first of a two-sided pair)
 // keep one order of additions at each size: whole tiles from 152 64 x 64 tiles
-// on, else 32 x 32 tiles with K split while the grid does not cover the SMs
-// and each rank keeps two K blocks.
+// on, else the small tiles.
 template <int NS, bool PRO, bool EPI>
 int pick_tile(const float* At, const float* B, float* C, int M, int N, int K, const Fused& f,
               const Epi& ep, int trans, bool solve, cudaStream_t st) {
@@ -618,7 +597,7 @@ int pick_tile(const float* At, const float* B, float* C, int M, int N, int K, co
                : run_fused<TileM<NS>, PRO, EPI, true>(At, B, C, M, N, K, KS, f, ep, trans, st);
   }
   const long tiles = (long)((M + 31) / 32) * ((N + 31) / 32);
-  while (KS < 8 && tiles * KS < NSM && K >= (solve ? 2 : 1) * BK * (KS * 2)) KS *= 2;
+  while (KS < 8 && tiles * KS < NSM && K >= 2 * BK * (KS * 2)) KS *= 2;
   const int kchunk = (((K + KS - 1) / KS) + BK - 1) / BK * BK;
   return launch_cluster(k_fused_small<NS, 32, 32, BK, 4, 2, PRO, EPI>, 32, 32, 128, 0, KS, At, B, C,
                         M, N, K, kchunk, f, ep, trans, st);

@@ -45,27 +45,60 @@ void transform_pair(int n, std::vector<double>& M, std::vector<double>& Mi) {
     }
 }
 
-__global__ void k_transpose_slices(const float* __restrict__ in, float* out, int R, int Cc,
-                                   const int* skip) {
+// out_z = in_z^T of R x C slices, 64 x 64 tiles of 256 threads, four elements a
+// load and a store (VEC: whole 16-byte groups on both sides), all of a
+// thread's loads in flight at once. Bound by HBM: one read and one write.
+template <bool VEC>
+__global__ void __launch_bounds__(256)
+k_transpose_slices(const float* __restrict__ in, float* out, int R, int C, const int* skip) {
   if (skip && *skip) return;
-  __shared__ float t[32][33];
-  const size_t so = (size_t)blockIdx.z * R * Cc;
-  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-  for (int i = threadIdx.y; i < 32; i += 8) {
-    const int r = r0 + i, c = c0 + threadIdx.x;
-    if (r < R && c < Cc) t[i][threadIdx.x] = in[so + (size_t)r * Cc + c];
+  __shared__ float t[64][65];
+  const size_t so = (size_t)blockIdx.z * R * C;
+  const int c0 = blockIdx.x * 64, r0 = blockIdx.y * 64;
+  const int q = threadIdx.x % 16 * 4, s = threadIdx.x / 16;
+  float v[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int r = r0 + s + 16 * i, c = c0 + q;
+    const float* src = in + so + (size_t)r * C + c;
+    if (VEC) {
+      const float4 x = r < R && c < C ? *reinterpret_cast<const float4*>(src)
+                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+      v[i][0] = x.x; v[i][1] = x.y; v[i][2] = x.z; v[i][3] = x.w;
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[i][e] = r < R && c + e < C ? src[e] : 0.f;
+    }
   }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) t[s + 16 * i][q + e] = v[i][e];
   __syncthreads();
-  for (int i = threadIdx.y; i < 32; i += 8) {
-    const int c = c0 + i, r = r0 + threadIdx.x;
-    if (r < R && c < Cc) out[so + (size_t)c * R + r] = t[threadIdx.x][i];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int c = c0 + s + 16 * i, r = r0 + q;
+    if (c >= C) break;
+    float* dst = out + so + (size_t)c * R + r;
+    if (VEC) {
+      if (r < R)
+        *reinterpret_cast<float4*>(dst) = make_float4(t[q][s + 16 * i], t[q + 1][s + 16 * i],
+                                                      t[q + 2][s + 16 * i], t[q + 3][s + 16 * i]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (r + e < R) dst[e] = t[q + e][s + 16 * i];
+    }
   }
 }
 
 int transpose_slices(const float* in, float* out, int R, int Cc, int n3, cudaStream_t st,
                      const int* skip = nullptr) {
-  dim3 grid((Cc + 31) / 32, (R + 31) / 32, n3);
-  k_transpose_slices<<<grid, dim3(32, 8), 0, st>>>(in, out, R, Cc, skip);
+  const dim3 grid((Cc + 63) / 64, (R + 63) / 64, n3);
+  const bool vec = R % 4 == 0 && Cc % 4 == 0 &&
+                   ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
+  if (vec) k_transpose_slices<true><<<grid, 256, 0, st>>>(in, out, R, Cc, skip);
+  else k_transpose_slices<false><<<grid, 256, 0, st>>>(in, out, R, Cc, skip);
   TC_CUDA(cudaGetLastError());
   return TC_OK;
 }
@@ -156,12 +189,14 @@ int cprod_epi(tc_plan* p, const float* X, float* Y, const Epi& ep, cudaStream_t 
     } else if (tct) {
       TC_TRY(launch_mode3_tc_lowp(X, lowop(p), p->dM, n3, P, rkind(p), ep.skip, err, st));
     } else if (x3(p)) {  // the exact FP32 pass, then the three planes
-      TC_TRY(launch_mode3(X, p->tmp2, p->dM, n3, P, mid, st));
+      TC_TRY(launch_mode3(X, p->tmp2, p->dMT, n3, P, mid, st));
       TC_TRY(launch_round(p->tmp2, p->lowX, P * n3, ROUND_BF16X3, st, ep.skip));
+    } else if (p->tmp3) {  // TF32: the operand is read K-major
+      TC_TRY(launch_mode3_tf32_kmajor(X, p->tmp3, p->dMT, n3, n2, s, ep.skip, st));
     } else {
-      TC_TRY(launch_mode3_lowp(X, p->tmp1, p->dM, n3, P, rkind(p) == ROUND_BF16, ep.skip, st));
+      TC_TRY(launch_mode3_bf16(X, p->tmp1, p->dMT, n3, P, ep.skip, st));
     }
-    if (p->tmp3) TC_TRY(transpose_slices(p->tmp1, p->tmp3, n2, s, n3, st, ep.skip));
+    if (p->tmp3 && tct) TC_TRY(transpose_slices(p->tmp1, p->tmp3, n2, s, n3, st, ep.skip));
     if (p->store_bf16) {  // BF16 slice products, read back by the BF16-input pass
       TC_TRY(launch_umma(*p->umf, p->tmp2, err, ep.skip, st, true));
       if (next_T)
@@ -172,9 +207,9 @@ int cprod_epi(tc_plan* p, const float* X, float* Y, const Epi& ep, cudaStream_t 
     TC_TRY(launch_umma(*p->umf, p->tmp2, err, ep.skip, st));
     if (p->two_sided) TC_TRY(right_factor(p, *p->umf2, (size_t)n1 * s * n3, err, ep.skip, st));
     return tct ? launch_mode3_tc(p->tmp2, Y, p->dMinv, n3, (size_t)n1 * s, ep, err, st, x3(p))
-               : launch_mode3(p->tmp2, Y, p->dMinv, n3, (size_t)n1 * s, ep, st);
+               : launch_mode3(p->tmp2, Y, p->dMinvT, n3, (size_t)n1 * s, ep, st);
   }
-  TC_TRY(launch_mode3(X, p->tmp1, p->dM, n3, (size_t)n2 * s, mid, st));
+  TC_TRY(launch_mode3(X, p->tmp1, p->dMT, n3, (size_t)n2 * s, mid, st));
   TC_TRY(launch_slice_gemm(p->AhT, p->tmp1, p->tmp2, n1, s, n2, n3, nullptr, nullptr, mid, st,
                            p->two_sided));
   const float* src = p->tmp2;
@@ -182,7 +217,7 @@ int cprod_epi(tc_plan* p, const float* X, float* Y, const Epi& ep, cudaStream_t 
     TC_TRY(launch_slice_gemm(p->tmp2, p->Bh, p->tmp1, n1, s, s, n3, nullptr, nullptr, mid, st));
     src = p->tmp1;
   }
-  return launch_mode3(src, Y, p->dMinv, n3, (size_t)n1 * s, ep, st);
+  return launch_mode3(src, Y, p->dMinvT, n3, (size_t)n1 * s, ep, st);
 }
 
 // Transform-domain products (ORTHODCT plans off the fused route): the
@@ -323,11 +358,12 @@ int adjoint_epi(tc_plan* p, const float* Y, float* X, const Epi& ep, cudaStream_
     } else if (tct) {
       TC_TRY(launch_mode3_tc_lowp(Y, lowop(p), p->dMinvT, n3, P, rkind(p), ep.skip, err, st));
     } else if (x3(p)) {
-      TC_TRY(launch_mode3(Y, p->tmp2, p->dMinvT, n3, P, mid, st));
+      TC_TRY(launch_mode3(Y, p->tmp2, p->dMinv, n3, P, mid, st));
       TC_TRY(launch_round(p->tmp2, p->lowX, P * n3, ROUND_BF16X3, st, ep.skip));
+    } else if (p->tmp3) {
+      TC_TRY(launch_mode3_tf32_kmajor(Y, p->tmp3, p->dMinv, n3, n1, s, ep.skip, st));
     } else {
-      TC_TRY(launch_mode3_lowp(Y, p->tmp1, p->dMinvT, n3, P, rkind(p) == ROUND_BF16, ep.skip,
-                               st));
+      TC_TRY(launch_mode3_bf16(Y, p->tmp1, p->dMinv, n3, P, ep.skip, st));
     }
     if (p->store_bf16) {  // BF16 slice products, read back by the BF16-input pass
       TC_TRY(launch_umma(*p->uma, p->tmp2, err, ep.skip, st, true));
@@ -336,13 +372,13 @@ int adjoint_epi(tc_plan* p, const float* Y, float* X, const Epi& ep, cudaStream_
                                      ep, err, st, after);
       return launch_mode3_tc_inb(p->tmp2, X, p->dMT, n3, (size_t)n2 * s, ep, err, st, after);
     }
-    if (p->tmp3) TC_TRY(transpose_slices(p->tmp1, p->tmp3, n1, s, n3, st, ep.skip));
+    if (p->tmp3 && tct) TC_TRY(transpose_slices(p->tmp1, p->tmp3, n1, s, n3, st, ep.skip));
     TC_TRY(launch_umma(*p->uma, p->tmp2, err, ep.skip, st));
     if (p->two_sided) TC_TRY(right_factor(p, *p->uma2, (size_t)n2 * s * n3, err, ep.skip, st));
     return tct ? launch_mode3_tc(p->tmp2, X, p->dMT, n3, (size_t)n2 * s, ep, err, st, x3(p), after)
-               : launch_mode3(p->tmp2, X, p->dMT, n3, (size_t)n2 * s, ep, st);
+               : launch_mode3(p->tmp2, X, p->dM, n3, (size_t)n2 * s, ep, st);
   }
-  TC_TRY(launch_mode3(Y, p->tmp1, p->dMinvT, n3, (size_t)n1 * s, mid, st));
+  TC_TRY(launch_mode3(Y, p->tmp1, p->dMinv, n3, (size_t)n1 * s, mid, st));
   TC_TRY(launch_slice_gemm(p->Ah, p->tmp1, p->tmp2, n2, s, n1, n3, nullptr, nullptr, mid, st,
                            p->two_sided));
   const float* src = p->tmp2;
@@ -350,7 +386,7 @@ int adjoint_epi(tc_plan* p, const float* Y, float* X, const Epi& ep, cudaStream_
     TC_TRY(launch_slice_gemm(p->tmp2, p->BhT, p->tmp1, n2, s, s, n3, nullptr, nullptr, mid, st));
     src = p->tmp1;
   }
-  return launch_mode3(src, X, p->dMT, n3, (size_t)n2 * s, ep, st);
+  return launch_mode3(src, X, p->dM, n3, (size_t)n2 * s, ep, st);
 }
 
 namespace {
@@ -421,13 +457,13 @@ int plan_build(tc_plan* p, const float* A, const float* B, cudaStream_t st) {
   TC_TRY(dalloc(&p->Ah, TA));
   TC_TRY(dalloc(&p->AhT, TA));
   Epi none;
-  TC_TRY(launch_mode3(A, p->Ah, p->dM, n3, (size_t)n1 * n2, none, st));
+  TC_TRY(launch_mode3(A, p->Ah, p->dMT, n3, (size_t)n1 * n2, none, st));
   TC_TRY(transpose_slices(p->Ah, p->AhT, n1, n2, n3, st));
   if (B) {
     const size_t TB = (size_t)n3 * s * s;
     TC_TRY(dalloc(&p->Bh, TB));
     TC_TRY(dalloc(&p->BhT, TB));
-    TC_TRY(launch_mode3(B, p->Bh, p->dM, n3, (size_t)s * s, none, st));
+    TC_TRY(launch_mode3(B, p->Bh, p->dMT, n3, (size_t)s * s, none, st));
     TC_TRY(transpose_slices(p->Bh, p->BhT, s, s, n3, st));
   }
   p->tmp_elems = p->Tx > p->Ty ? p->Tx : p->Ty;
@@ -666,7 +702,7 @@ extern "C" int tc_transform(tc_plan* p, int which, const float* in, float* out, 
   // TC_TUBE_MIN_N3 (three BF16 planes for TC_BF16X3), the FP32 pass otherwise
   if (lowp(p) && p->n3 > TC_TUBE_MIN_N3)
     return launch_mode3_tc(in, out, T, p->n3, P, ep, p->dev_err, st, x3(p));
-  return launch_mode3(in, out, T, p->n3, P, ep, st);
+  return launch_mode3(in, out, transposed(p, T), p->n3, P, ep, st);
 }
 
 extern "C" int tc_transform_dual(tc_plan* p, int which, const float* in, void* out, size_t P,

@@ -190,7 +190,7 @@ int lsqr_enqueue(tc_plan* p, const LsqrArgs& a, cudaStream_t st) {
     Epi none;
     return tct ? launch_mode3_tc(in, out, T, p->n3, P, none, p->dev_err, st,
                                  p->opts.precision == TC_BF16X3)
-               : launch_mode3(in, out, T, p->n3, P, none, st);
+               : launch_mode3(in, out, transposed(p, T), p->n3, P, none, st);
   };
   if (td) {
     TC_TRY(mode3(a.C, p->lsqr_Ct, p->dM, p->Ty / p->n3));

@@ -146,6 +146,33 @@ __device__ __forceinline__ bool reduce_finish(float v, const Red& red) {
   return reduce_finish_n(v, red, bid, nblk);
 }
 
+// The last CTA's part of such a reduction, by threads 0..127 standing for 128 V
+// (thread t is threads t, t + 128, ..; every thread of the CTA calls it): the
+// same sums in the same order as reduce_finish_n over 128 V threads.
+template <int V>
+__device__ __forceinline__ void sum_partials(const Red& red, size_t nblk) {
+  __shared__ double sh_d[4 * V];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  if (tid < 128) {
+#pragma unroll
+    for (int q = 0; q < V; ++q) {
+      double acc = 0.0;
+      for (size_t i = tid + 128 * q; i < nblk; i += 128 * V) acc += __ldcg(red.partials + i);
+      acc = warp_sum(acc);
+      if (lane == 0) sh_d[4 * q + w] = acc;
+    }
+  }
+  __syncthreads();
+  if (tid < 32) {
+    const double t = warp_sum(lane < 4 * V ? sh_d[lane] : 0.0);
+    if (tid == 0) {
+      if (red.status && !isfinite(t)) *red.status = TC_ENONFINITE;
+      *red.out = red.sqrt_out ? sqrt(t) : t;
+      *red.ticket = 0u;
+    }
+  }
+}
+
 // LSQR step scalars (Algorithm 6 steps (c)-(g), 0-based step j):
 //   rho = hypot(rhobar_j, beta_{j+1}), c = rhobar_j/rho, s = beta_{j+1}/rho,
 //   theta = s alpha_{j+1}, rhobar_{j+1} = c alpha_{j+1},

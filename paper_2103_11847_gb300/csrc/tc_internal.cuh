@@ -193,18 +193,28 @@ int cprod2_init();
 int launch_cprod2(const float* At, const float* X, const float* B, float* Y, int M, int K,
                   int N, int nslices, const float* pro, const float* epi, const Epi& ep,
                   const LsqrStep& step, cudaStream_t st);
-// transform.cu: out[k][p] = ca * sum_l T[k][l] in[l][p] + cp * prev[k][p] over P pixels.
-int launch_mode3(const float* in, float* out, const float* T_dev, int n3, size_t P,
+// mode3.cu: out[k][p] = ca * sum_l T[k][l] in[l][p] + cp * prev[k][p] over P
+// pixels, T given by its transpose Tt (device, n3 x n3).
+int launch_mode3(const float* in, float* out, const float* Tt, int n3, size_t P,
                  const Epi& ep, cudaStream_t st);
-// The same transform writing the operand of a tensor-core GEMM: BF16, or FP32
-// rounded to TF32 (bf16 = 0). No epilogue.
-int launch_mode3_lowp(const float* in, void* out, const float* T_dev, int n3, size_t P,
-                      int bf16, const int* skip, cudaStream_t st);
+// The same transform writing the BF16 operand of a tensor-core GEMM. No epilogue.
+int launch_mode3_bf16(const float* in, void* out, const float* Tt, int n3, size_t P,
+                      const int* skip, cudaStream_t st);
+// The TF32 operand K-major: pixels are rows x cols row-major, out is cols x rows
+// a slice.
+int launch_mode3_tf32_kmajor(const float* in, float* out, const float* Tt, int n3, int rows,
+                             int cols, const int* skip, cudaStream_t st);
+int mode3_init();
+// The transpose of one of the plan's transforms dM, dMinv, dMinvT, dMT.
+inline const float* transposed(const tc_plan* p, const float* T) {
+  return T == p->dM ? p->dMT : T == p->dMT ? p->dM : T == p->dMinv ? p->dMinvT : p->dMinv;
+}
+// transform.cu
 // GEMM operand types of the tensor-core forms: TF32 (in FP32 storage), BF16,
 // and three BF16 planes (plane q of n values at out + q n) for the
 // FP32-level form.
 enum RoundKind { ROUND_TF32 = 0, ROUND_BF16 = 1, ROUND_BF16X3 = 2 };
-// Tensor-core forms of launch_mode3 / launch_mode3_lowp (tcgen05, operands
+// Tensor-core forms of launch_mode3 / launch_mode3_bf16 (tcgen05, operands
 // split into BF16 planes: two, relative error near 2^-16 a term, for the TF32
 // and BF16 forms; three (split3 / ROUND_BF16X3), near 2^-27, for the
 // FP32-level form). *err is set to TC_ETIMEOUT if the bounded wait for the

@@ -1,13 +1,8 @@
-// Mode-3 transform pass for n3 > TC_MAX_FUSED (Remark 2.1: X~ = X x_3 T with
-// T one of M, M^{-1}, M^{-T}, M^T): out[k][p] = ca * sum_l T[k][l] in[l][p]
-// + cp * prev[k][p], with the fused reduction of the epilogue. Each CTA owns
-// 128 consecutive pixels p of every slice: warp w computes the KPW contiguous
-// outputs k = w*KPW .. w*KPW + KPW - 1 (coefficients read as float4
-// broadcasts) and lane q the pixels 4q..4q+3. T is staged in shared memory
-// once. The CTA's whole input block (every slice of its 128 pixels, 32 KB at
-// n3 = 64) is requested at once with cp.async in groups of 16 slices, and
-// each group is consumed as it lands, so a CTA keeps its whole input in
-// flight. HBM traffic is one read of `in` (and `prev`) and one write of `out`.
+// Mode-3 transform passes on the tensor cores (Remark 2.1: X~ = X x_3 T with T one
+// of M, M^{-1}, M^{-T}, M^T), for the precision forms above TC_TUBE_MIN_N3: out[k][p]
+// = ca * sum_l T[k][l] in[l][p] + cp * prev[k][p], with the fused reduction of the
+// epilogue; and the elementwise rounding to a GEMM's input type. (mode3.cu has
+// the FFMA pass of the other plans.)
 #include <cuda_bf16.h>
 
 #include "tc_device.cuh"
@@ -27,183 +22,11 @@ __device__ __forceinline__ float round_tf32(float x) {
   return __uint_as_float(r);
 }
 
-constexpr int PB = 128;  // pixels per CTA
-constexpr int LC = 16;   // input slices per cp.async group
-
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem, bool valid) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
   const int n = valid ? 16 : 0;  // zero-fill when out of range
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(s), "l"(gmem), "r"(n)
                : "memory");
-}
-
-// Dynamic shared memory of k_mode3<KPW, .>: T^T (8 KPW x 8 KPW) and the whole
-// input block (8 KPW slices x PB pixels).
-template <int KPW>
-constexpr size_t mode3_smem() { return (size_t)(8 * KPW) * (8 * KPW + PB) * sizeof(float); }
-
-__device__ __forceinline__ void cp_wait_upto(int n) {  // at most n groups pending
-  if (n <= 0) asm volatile("cp.async.wait_group 0;" ::: "memory");
-  else if (n == 1) asm volatile("cp.async.wait_group 1;" ::: "memory");
-  else if (n == 2) asm volatile("cp.async.wait_group 2;" ::: "memory");
-  else asm volatile("cp.async.wait_group 3;" ::: "memory");
-}
-
-template <int KPW, int OUT>
-__global__ void __launch_bounds__(256, 3)
-k_mode3(const float* __restrict__ in, void* out_v, const float* __restrict__ T, int n3,
-        size_t P, Epi ep) {
-  if (ep.skip && *ep.skip) return;
-  // ts: T transposed (ts[l][k] = T[k][l]), loaded once; xs: the CTA's whole
-  // input block, every slice of its PB pixels, requested at once in groups of
-  // LC slices so that all of it is in flight while the first groups compute
-  extern __shared__ __align__(16) float m3_smem[];
-  float(*ts)[8 * KPW] = reinterpret_cast<float(*)[8 * KPW]>(m3_smem);
-  float(*xs)[PB] = reinterpret_cast<float(*)[PB]>(m3_smem + (8 * KPW) * (8 * KPW));
-  __shared__ float sh_coef[2];
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const size_t p0 = (size_t)blockIdx.x * PB;
-  // float4 path: whole groups of 4 pixels and 16-byte aligned tensors
-  auto al16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
-  const bool vec = (P % 4 == 0) && al16(in) && al16(out_v) && (!ep.prev || al16(ep.prev)) &&
-                   (!ep.red.other || al16(ep.red.other));
-  float acc[KPW][4];
-#pragma unroll
-  for (int q = 0; q < KPW; ++q)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) acc[q][e] = 0.f;
-
-  const int nch = (n3 + LC - 1) / LC;  // <= 4 (n3 <= 64)
-  for (int c = 0; c < nch; ++c) {
-    const int l0 = c * LC, lc_n = min(LC, n3 - l0);
-    if (vec) {
-      for (int idx = tid; idx < LC * PB / 4; idx += 256) {
-        const int lc = idx / (PB / 4), px = (idx % (PB / 4)) * 4;
-        const size_t p = p0 + px;
-        if (lc < lc_n) {
-          const bool ok = p < P;
-          cp_async16(&xs[l0 + lc][px], ok ? in + (size_t)(l0 + lc) * P + p : in, ok);
-        }
-      }
-    } else {
-      for (int idx = tid; idx < LC * PB; idx += 256) {
-        const int lc = idx / PB, px = idx % PB;
-        const size_t p = p0 + px;
-        if (lc < lc_n) xs[l0 + lc][px] = p < P ? __ldg(in + (size_t)(l0 + lc) * P + p) : 0.f;
-      }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  }
-  for (int idx = tid; idx < n3 * 8 * KPW; idx += 256) {
-    const int l = idx / (8 * KPW), k = idx % (8 * KPW);
-    ts[l][k] = (k < n3) ? __ldg(T + (size_t)k * n3 + l) : 0.f;
-  }
-  for (int c = 0; c < nch; ++c) {
-    cp_wait_upto(nch - 1 - c);  // this thread's copies of group c have landed
-    __syncthreads();            // everyone's, and T
-    const int l0 = c * LC, lc_n = min(LC, n3 - l0);
-    for (int lc = 0; lc < lc_n; ++lc) {
-      const float4 x = *reinterpret_cast<const float4*>(&xs[l0 + lc][lane * 4]);
-      float t[KPW];  // warp w owns the contiguous outputs k = w*KPW .. w*KPW + KPW - 1
-      if (KPW % 4 == 0) {
-#pragma unroll
-        for (int q = 0; q < KPW; q += 4) {
-          const float4 tv = *reinterpret_cast<const float4*>(&ts[l0 + lc][w * KPW + q]);
-          t[q] = tv.x; t[q + 1] = tv.y; t[q + 2] = tv.z; t[q + 3] = tv.w;
-        }
-      } else {
-#pragma unroll
-        for (int q = 0; q < KPW; ++q) t[q] = ts[l0 + lc][w * KPW + q];
-      }
-#pragma unroll
-      for (int q = 0; q < KPW; ++q) {
-        acc[q][0] = fmaf(t[q], x.x, acc[q][0]);
-        acc[q][1] = fmaf(t[q], x.y, acc[q][1]);
-        acc[q][2] = fmaf(t[q], x.z, acc[q][2]);
-        acc[q][3] = fmaf(t[q], x.w, acc[q][3]);
-      }
-    }
-  }
-
-  if (OUT != OUT_F32) {  // operand of a tensor-core GEMM: store only
-#pragma unroll
-    for (int q = 0; q < KPW; ++q) {
-      const int k = w * KPW + q;
-      if (k >= n3) continue;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const size_t p = p0 + lane * 4 + e;
-        if (p < P) {
-          const size_t idx = (size_t)k * P + p;
-          if (OUT == OUT_BF16)
-            static_cast<__nv_bfloat16*>(out_v)[idx] = __float2bfloat16_rn(acc[q][e]);
-          else
-            static_cast<float*>(out_v)[idx] = round_tf32(acc[q][e]);
-        }
-      }
-    }
-    return;
-  }
-  float* out = static_cast<float*>(out_v);
-  coef_compute(ep.coef, sh_coef);
-  __syncthreads();
-  const float ca = sh_coef[0], cp = sh_coef[1];
-  float local = 0.f;
-#pragma unroll
-  for (int q = 0; q < KPW; ++q) {
-    const int k = w * KPW + q;
-    if (k >= n3) continue;
-    const size_t pb = p0 + lane * 4;
-    if (vec && pb + 4 <= P) {
-      const size_t idx = (size_t)k * P + pb;
-      float4 o = make_float4(ca * acc[q][0], ca * acc[q][1], ca * acc[q][2], ca * acc[q][3]);
-      if (ep.prev) {
-        const float4 pv = *reinterpret_cast<const float4*>(ep.prev + idx);
-        o.x = fmaf(cp, pv.x, o.x); o.y = fmaf(cp, pv.y, o.y);
-        o.z = fmaf(cp, pv.z, o.z); o.w = fmaf(cp, pv.w, o.w);
-      }
-      *reinterpret_cast<float4*>(out + idx) = o;
-      if (ep.red.out) {
-        if (ep.red.other) {
-          const float4 ov = *reinterpret_cast<const float4*>(ep.red.other + idx);
-          local = fmaf(o.x, ov.x, fmaf(o.y, ov.y, fmaf(o.z, ov.z, fmaf(o.w, ov.w, local))));
-        } else {
-          local = fmaf(o.x, o.x, fmaf(o.y, o.y, fmaf(o.z, o.z, fmaf(o.w, o.w, local))));
-        }
-      }
-      continue;
-    }
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const size_t p = pb + e;
-      if (p < P) {
-        const size_t idx = (size_t)k * P + p;
-        float o = ca * acc[q][e];
-        if (ep.prev) o = fmaf(cp, ep.prev[idx], o);
-        out[idx] = o;
-        if (ep.red.out) local = fmaf(o, ep.red.other ? ep.red.other[idx] : o, local);
-      }
-    }
-  }
-  if (ep.red.out) reduce_finish(local, ep.red);
-}
-
-template <int KPW, int OUT>
-int run(const float* in, void* out, const float* T, int n3, size_t P, const Epi& ep,
-        cudaStream_t st) {
-  const size_t blocks = (P + PB - 1) / PB;
-  k_mode3<KPW, OUT><<<(unsigned)blocks, 256, mode3_smem<KPW>(), st>>>(in, out, T, n3, P, ep);
-  TC_CUDA(cudaGetLastError());
-  return TC_OK;
-}
-
-template <int OUT>
-int pick(const float* in, void* out, const float* T, int n3, size_t P, const Epi& ep,
-         cudaStream_t st) {
-  if (n3 <= 8) return run<1, OUT>(in, out, T, n3, P, ep, st);
-  if (n3 <= 16) return run<2, OUT>(in, out, T, n3, P, ep, st);
-  if (n3 <= 32) return run<4, OUT>(in, out, T, n3, P, ep, st);
-  return run<8, OUT>(in, out, T, n3, P, ep, st);
 }
 
 // Elementwise rounding to the GEMM input type; four elements per thread and
@@ -1336,31 +1159,6 @@ int run_tube_tma(const float* in, void* out, const float* T, int n3, size_t P, c
 
 }  // namespace
 
-int launch_mode3(const float* in, float* out, const float* T_dev, int n3, size_t P,
-                 const Epi& ep, cudaStream_t st) {
-  TC_CHECK(n3 >= 1 && n3 <= TC_MAX_N3);
-  return pick<OUT_F32>(in, out, T_dev, n3, P, ep, st);
-}
-
-int launch_mode3_lowp(const float* in, void* out, const float* T_dev, int n3, size_t P,
-                      int bf16, const int* skip, cudaStream_t st) {
-  TC_CHECK(n3 >= 1 && n3 <= TC_MAX_N3);
-  Epi ep;
-  ep.skip = skip;
-  return bf16 ? pick<OUT_BF16>(in, out, T_dev, n3, P, ep, st)
-              : pick<OUT_TF32>(in, out, T_dev, n3, P, ep, st);
-}
-
-namespace {
-template <int KPW>
-int init_kpw() {
-  for (auto fn : {k_mode3<KPW, OUT_F32>, k_mode3<KPW, OUT_BF16>, k_mode3<KPW, OUT_TF32>})
-    TC_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)mode3_smem<KPW>()));
-  return TC_OK;
-}
-}  // namespace
-
 namespace {
 
 // persistent grid: tube_ctas(ns) CTAs a SM, no more than one a tile
@@ -1513,10 +1311,6 @@ int transform_init() {
   int dev = 0;
   TC_CUDA(cudaGetDevice(&dev));
   TC_CUDA(cudaDeviceGetAttribute(&g_tube_sms, cudaDevAttrMultiProcessorCount, dev));
-  TC_TRY(init_kpw<1>());
-  TC_TRY(init_kpw<2>());
-  TC_TRY(init_kpw<4>());
-  TC_TRY(init_kpw<8>());
   return TC_OK;
 }
 
