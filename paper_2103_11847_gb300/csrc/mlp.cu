@@ -7,6 +7,11 @@
 // Parameters are one flat FP32 vector, W1 (36 x 64, row-major in x out), b1,
 // W2 (64 x 64), b2, W3 (64 x 2), b3. The loss is (1/2B) sum (out - t)^2. All
 // reductions over the batch run in a fixed order, so training is deterministic.
+//
+// A training step is two launches, each started while the last one finishes
+// (programmatic dependent launch): the samples' pass and the gradients with
+// the Adam step. As four launches (forward, backward, gradients as chains of
+// global loads, Adam) a step of 256 samples took 33 us, now 12.
 #include <cuda_bf16.h>
 
 #include <new>
@@ -27,114 +32,241 @@ __device__ __forceinline__ float gelu_d(float z) {
   return 0.5f * (1.f + erff(z * 0.70710678118654752f)) + z * 0.3989422804014327f * expf(-0.5f * z * z);
 }
 
-// One CTA of 64 threads per sample: z1, h1, z2, h2, out (saved for backward).
-__global__ void __launch_bounds__(NH)
-k_mlp_fwd(const float* __restrict__ X, int B, const __nv_bfloat16* __restrict__ Wb,
-          const float* __restrict__ theta, float* Z1, float* H1, float* Z2, float* H2, float* OUT) {
-  __shared__ float x[NI], h1[NH], h2[NH];
-  const int b = blockIdx.x, j = threadIdx.x;
-  if (b >= B) return;
-  for (int i = j; i < NI; i += NH) x[i] = X[(size_t)b * NI + i];
+// The pass over samples, four a CTA of 256 threads (64 a sample): forward, and
+// with targets (T non-null) the loss and the backward pass through the
+// activations, D = (out - t) / B, dZ2 = (D W3^T) * gelu'(z2), dZ1 = (dZ2 W2^T) *
+// gelu'(z1).
+//
+// Bound: latency (a batch of 256 is 10 MFLOP; every sum over inputs is one chain
+// of at most 64 FMAs). The BF16 weights are staged in shared memory once a CTA
+// with 16-byte copies; W2's rows are 66 values apart, so that both its columns
+// (forward) and its rows (backward) are read without bank conflicts. z1 and z2
+// stay in registers.
+constexpr int SPC = 4;           // samples a CTA
+constexpr int W2S = NH + 2;      // row stride of W2 in shared memory
+
+__global__ void __launch_bounds__(SPC * NH)
+k_mlp_samples(const float* __restrict__ X, const float* __restrict__ T, int B,
+              const __nv_bfloat16* Wb, const float* theta, float* H1, float* H2, float* OUT,
+              float* D, float* dZ1, float* dZ2, float* lossb) {
+  __shared__ __align__(16) __nv_bfloat16 w1[NI * NH];
+  __shared__ __align__(16) __nv_bfloat16 w2[NH * W2S];
+  __shared__ __align__(16) __nv_bfloat16 w3[NH * NO];
+  __shared__ float xs[SPC][NI], h1s[SPC][NH], h2s[SPC][NH], dz2s[SPC][NH], ds[SPC][NO];
+  const int tid = threadIdx.x, q = tid / NH, j = tid % NH;
+  const int b = blockIdx.x * SPC + q;
+  const bool live = b < B;
+  for (int i = tid; i < SPC * NI; i += SPC * NH) {
+    const int bb = blockIdx.x * SPC + i / NI;
+    xs[i / NI][i % NI] = bb < B ? X[(size_t)blockIdx.x * SPC * NI + i] : 0.f;
+  }
+  pdl_trigger();
+  pdl_wait();  // the weights are the last step's
+  for (int i = tid; i < NI * NH / 8; i += SPC * NH)
+    reinterpret_cast<uint4*>(w1)[i] = reinterpret_cast<const uint4*>(Wb + OW1)[i];
+  for (int i = tid; i < NH * NH / 8; i += SPC * NH) {
+    const uint4 v = reinterpret_cast<const uint4*>(Wb + OW2)[i];
+    uint32_t* d = reinterpret_cast<uint32_t*>(w2 + (i / (NH / 8)) * W2S + (i % (NH / 8)) * 8);
+    d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
+  }
+  if (tid < NH * NO / 8) reinterpret_cast<uint4*>(w3)[tid] = reinterpret_cast<const uint4*>(Wb + OW3)[tid];
+  const float bias1 = theta[OB1 + j], bias2 = theta[OB2 + j];
   __syncthreads();
-  float z = theta[OB1 + j];
-  for (int i = 0; i < NI; ++i) z = fmaf(x[i], __bfloat162float(Wb[OW1 + i * NH + j]), z);
-  h1[j] = gelu(z);
-  if (Z1) { Z1[(size_t)b * NH + j] = z; H1[(size_t)b * NH + j] = h1[j]; }
+  float z1 = bias1;
+#pragma unroll
+  for (int i = 0; i < NI; ++i) z1 = fmaf(xs[q][i], __bfloat162float(w1[i * NH + j]), z1);
+  const float h1 = gelu(z1);
+  h1s[q][j] = h1;
+  if (H1 && live) H1[(size_t)b * NH + j] = h1;
   __syncthreads();
-  z = theta[OB2 + j];
-  for (int i = 0; i < NH; ++i) z = fmaf(h1[i], __bfloat162float(Wb[OW2 + i * NH + j]), z);
-  h2[j] = gelu(z);
-  if (Z2) { Z2[(size_t)b * NH + j] = z; H2[(size_t)b * NH + j] = h2[j]; }
+  float z2 = bias2;
+#pragma unroll
+  for (int i = 0; i < NH; ++i) z2 = fmaf(h1s[q][i], __bfloat162float(w2[i * W2S + j]), z2);
+  const float h2 = gelu(z2);
+  h2s[q][j] = h2;
+  if (H2 && live) H2[(size_t)b * NH + j] = h2;
   __syncthreads();
   if (j < NO) {
     float o = theta[OB3 + j];
-    for (int i = 0; i < NH; ++i) o = fmaf(h2[i], __bfloat162float(Wb[OW3 + i * NO + j]), o);
-    OUT[(size_t)b * NO + j] = o;
-  }
-}
-
-// Backward through the activations, one CTA per sample: D = (out - t) / B,
-// dZ2 = (D W3^T) * gelu'(z2), dZ1 = (dZ2 W2^T) * gelu'(z1); per-sample loss.
-__global__ void __launch_bounds__(NH)
-k_mlp_bwd_act(const float* __restrict__ T, int B, const __nv_bfloat16* __restrict__ Wb,
-              const float* Z1, const float* Z2, const float* OUT, float* D, float* dZ1,
-              float* dZ2, float* lossb) {
-  __shared__ float d[NO], dz2[NH];
-  const int b = blockIdx.x, j = threadIdx.x;
-  if (j < NO) {
-    const float r = OUT[(size_t)b * NO + j] - T[(size_t)b * NO + j];
-    d[j] = r / B;
-    D[(size_t)b * NO + j] = r / B;
-  }
-  if (j == 0) {
-    float l = 0.f;
-    for (int o = 0; o < NO; ++o) {
-      const float r = OUT[(size_t)b * NO + o] - T[(size_t)b * NO + o];
-      l = fmaf(r, r, l);
+#pragma unroll
+    for (int i = 0; i < NH; ++i) o = fmaf(h2s[q][i], __bfloat162float(w3[i * NO + j]), o);
+    if (OUT && live) OUT[(size_t)b * NO + j] = o;
+    if (T) {
+      const float r = live ? o - T[(size_t)b * NO + j] : 0.f;
+      ds[q][j] = r / B;
+      if (live) D[(size_t)b * NO + j] = r / B;
+      float l = 0.f;  // threads 0 and 1 of the sample are neighbours in one warp
+#pragma unroll
+      for (int k = 0; k < NO; ++k) {
+        const float rk = __shfl_sync((1u << NO) - 1, r, k, NO);
+        l = fmaf(rk, rk, l);
+      }
+      if (j == 0 && live) lossb[b] = 0.5f * l / B;
     }
-    lossb[b] = 0.5f * l / B;
   }
+  if (!T) return;
   __syncthreads();
   float g = 0.f;
-  for (int o = 0; o < NO; ++o) g = fmaf(d[o], __bfloat162float(Wb[OW3 + j * NO + o]), g);
-  dz2[j] = g * gelu_d(Z2[(size_t)b * NH + j]);
-  dZ2[(size_t)b * NH + j] = dz2[j];
+#pragma unroll
+  for (int o = 0; o < NO; ++o) g = fmaf(ds[q][o], __bfloat162float(w3[j * NO + o]), g);
+  const float dz2 = g * gelu_d(z2);
+  dz2s[q][j] = dz2;
+  if (live) dZ2[(size_t)b * NH + j] = dz2;
   __syncthreads();
   g = 0.f;
-  for (int k = 0; k < NH; ++k) g = fmaf(dz2[k], __bfloat162float(Wb[OW2 + j * NH + k]), g);
-  dZ1[(size_t)b * NH + j] = g * gelu_d(Z1[(size_t)b * NH + j]);
+#pragma unroll
+  for (int k = 0; k < NH; ++k) g = fmaf(dz2s[q][k], __bfloat162float(w2[j * W2S + k]), g);
+  if (live) dZ1[(size_t)b * NH + j] = g * gelu_d(z1);
 }
 
-// Weight gradients, one thread per parameter, batch summed in order.
-__global__ void k_mlp_bwd_w(const float* __restrict__ X, int B, const float* H1, const float* H2,
-                            const float* D, const float* dZ1, const float* dZ2,
-                            const float* lossb, float* grad, float* loss) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p == 0 && loss) {
-    float l = 0.f;
-    for (int b = 0; b < B; ++b) l += lossb[b];
-    *loss = l;
+// Adam (bias-corrected) on parameter p; refreshes its BF16 copy.
+struct Adam {
+  float* theta = nullptr;  // null: gradients only
+  float* m = nullptr;
+  float* v = nullptr;
+  __nv_bfloat16* Wb = nullptr;
+  int t = 0;
+  float lr = 0.f;
+};
+
+// A parameter's Adam state, read before its gradient is summed so that the
+// reads and the bias corrections are off the end of the launch.
+struct AdamState {
+  float th = 0.f, m = 0.f, v = 0.f;
+};
+
+__device__ __forceinline__ AdamState adam_read(const Adam& a, int p, bool live) {
+  AdamState s;
+  if (a.theta && live) {
+    s.th = a.theta[p];
+    s.m = a.m[p];
+    s.v = a.v[p];
   }
-  if (p >= MLP_NPARAMS) return;
-  float s = 0.f;
-  if (p < OB1) {
-    const int i = p / NH, j = p % NH;
-    for (int b = 0; b < B; ++b) s = fmaf(X[(size_t)b * NI + i], dZ1[(size_t)b * NH + j], s);
-  } else if (p < OW2) {
-    const int j = p - OB1;
-    for (int b = 0; b < B; ++b) s += dZ1[(size_t)b * NH + j];
-  } else if (p < OB2) {
-    const int i = (p - OW2) / NH, j = (p - OW2) % NH;
-    for (int b = 0; b < B; ++b) s = fmaf(H1[(size_t)b * NH + i], dZ2[(size_t)b * NH + j], s);
-  } else if (p < OW3) {
-    const int j = p - OB2;
-    for (int b = 0; b < B; ++b) s += dZ2[(size_t)b * NH + j];
-  } else if (p < OB3) {
-    const int i = (p - OW3) / NO, o = (p - OW3) % NO;
-    for (int b = 0; b < B; ++b) s = fmaf(H2[(size_t)b * NH + i], D[(size_t)b * NO + o], s);
-  } else {
-    const int o = p - OB3;
-    for (int b = 0; b < B; ++b) s += D[(size_t)b * NO + o];
-  }
-  grad[p] = s;
+  return s;
 }
 
-// Adam (bias-corrected); refreshes the BF16 copies of the weight matrices.
-__global__ void k_adam(float* theta, const float* grad, float* m, float* v, int t, float lr,
-                       __nv_bfloat16* Wb) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= MLP_NPARAMS) return;
+__device__ __forceinline__ void put_grad(int p, float g, float* grad, const Adam& a,
+                                         const AdamState& s, float c1, float c2) {
+  if (!a.theta) {
+    grad[p] = g;
+    return;
+  }
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  const float g = grad[p];
-  const float mm = b1 * m[p] + (1.f - b1) * g;
-  const float vv = b2 * v[p] + (1.f - b2) * g * g;
-  m[p] = mm;
-  v[p] = vv;
-  const float mh = mm / (1.f - powf(b1, (float)t));
-  const float vh = vv / (1.f - powf(b2, (float)t));
-  const float th = theta[p] - lr * mh / (sqrtf(vh) + eps);
-  theta[p] = th;
-  Wb[p] = __float2bfloat16_rn(th);
+  const float mm = b1 * s.m + (1.f - b1) * g;
+  const float vv = b2 * s.v + (1.f - b2) * g * g;
+  a.m[p] = mm;
+  a.v[p] = vv;
+  const float mh = mm / c1;
+  const float vh = vv / c2;
+  const float th = s.th - a.lr * mh / (sqrtf(vh) + eps);
+  a.theta[p] = th;
+  a.Wb[p] = __float2bfloat16_rn(th);
+}
+
+// Parameter gradients, each one chain over the batch in order, and the Adam
+// step on them. A CTA of 64 threads owns 4 rows x 32 columns of [W1; b1] (37
+// rows, the last against ones) or [W2; b2] (65 rows), two rows a thread; the
+// last CTA owns W3, b3 and the loss. The columns of dZ and of the layer's input
+// come through shared memory in chunks of GB samples, the next chunk in flight
+// (cp.async) while this one is summed: the sums are chains of FMAs on
+// shared-memory operands instead of chains of global loads.
+constexpr int GB = 128, GT = 64;
+constexpr int GR1 = (NI + 1 + 3) / 4, GR2 = (NH + 1 + 3) / 4;  // row groups of the two layers
+constexpr int GCTAS = 2 * GR1 + 2 * GR2 + 1;
+
+__device__ __forceinline__ void cp_async(float* dst, const float* src, int bytes) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  if (bytes == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+}
+
+__global__ void __launch_bounds__(GT)
+k_mlp_grad(const float* __restrict__ X, int B, const float* H1, const float* H2, const float* D,
+           const float* dZ1, const float* dZ2, const float* lossb, float* grad, float* loss,
+           Adam a) {
+  __shared__ __align__(16) float vs[2][GB][32];
+  __shared__ __align__(16) float us[2][GB][4];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  pdl_trigger();
+  const float c1 = 1.f - powf(0.9f, (float)a.t), c2 = 1.f - powf(0.999f, (float)a.t);
+  pdl_wait();  // the activations and their gradients are the samples' pass's
+  const int nch = (B + GB - 1) / GB;
+  if (blockIdx.x == GCTAS - 1) {  // W3 (64 x 2), b3, loss: H2 in two halves of 32 columns
+    float s[NO] = {0.f, 0.f}, t = 0.f;
+    const AdamState q0 = adam_read(a, OW3 + tid * NO, true);
+    const AdamState q1 = adam_read(a, OW3 + tid * NO + 1, true);
+    const AdamState q3 = adam_read(a, OB3 + tid, tid < NO);
+    for (int b0 = 0; b0 < B; b0 += GB) {
+      const int nb = min(GB, B - b0);
+      __syncthreads();
+      for (int i = tid; i < nb * (NH / 4); i += GT) {
+        const int r = i / (NH / 4), c = (i % (NH / 4)) * 4;
+        cp_async(&vs[c / 32][r][c % 32], H2 + (size_t)(b0 + r) * NH + c, 16);
+      }
+      for (int i = tid; i < nb; i += GT) {
+        cp_async(&us[0][i][0], D + (size_t)(b0 + i) * NO, 4);
+        cp_async(&us[0][i][1], D + (size_t)(b0 + i) * NO + 1, 4);
+        cp_async(&us[0][i][2], lossb + b0 + i, 4);
+      }
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncthreads();
+#pragma unroll 8
+      for (int r = 0; r < nb; ++r) {
+        const float h = vs[w][r][lane];
+        s[0] = fmaf(h, us[0][r][0], s[0]);
+        s[1] = fmaf(h, us[0][r][1], s[1]);
+        if (tid < 3) t += us[0][r][tid];  // b3[0], b3[1], loss
+      }
+    }
+    put_grad(OW3 + tid * NO, s[0], grad, a, q0, c1, c2);
+    put_grad(OW3 + tid * NO + 1, s[1], grad, a, q1, c1, c2);
+    if (tid < NO) put_grad(OB3 + tid, t, grad, a, q3, c1, c2);
+    if (tid == NO && loss) *loss = t;
+    return;
+  }
+  const bool second = blockIdx.x >= 2 * GR1;
+  const int g = second ? blockIdx.x - 2 * GR1 : blockIdx.x;
+  const int rows = second ? NH : NI, r0 = (g / 2) * 4, c0 = (g % 2) * 32;
+  const float* U = second ? H1 : X;      // the layer's input, rows values a sample
+  const float* V = second ? dZ2 : dZ1;   // its output's gradient
+  auto issue = [&](int c) {
+    const int b0 = c * GB, nb = min(GB, B - b0);
+    for (int i = tid; i < nb * 8; i += GT)
+      cp_async(&vs[c & 1][i / 8][(i % 8) * 4], V + (size_t)(b0 + i / 8) * NH + c0 + (i % 8) * 4, 16);
+    for (int i = tid; i < nb * 4; i += GT) {
+      const int r = i / 4, k = r0 + i % 4;
+      if (k < rows) cp_async(&us[c & 1][r][i % 4], U + (size_t)(b0 + r) * rows + k, 4);
+      else us[c & 1][r][i % 4] = 1.f;  // the bias row
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  issue(0);
+  // [W; b] is contiguous: row k, column j at k NH + j, the bias as row `rows`
+  const int k = r0 + 2 * w, p = (second ? OW2 : OW1) + k * NH + c0 + lane;
+  const AdamState q0 = adam_read(a, p, k <= rows), q1 = adam_read(a, p + NH, k + 1 <= rows);
+  float s0 = 0.f, s1 = 0.f;
+  for (int c = 0; c < nch; ++c) {
+    if (c + 1 < nch) {
+      issue(c + 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+    const int nb = min(GB, B - c * GB);
+#pragma unroll 16
+    for (int r = 0; r < nb; ++r) {
+      const float v = vs[c & 1][r][lane];
+      const float2 u = *reinterpret_cast<const float2*>(&us[c & 1][r][2 * w]);
+      s0 = fmaf(u.x, v, s0);
+      s1 = fmaf(u.y, v, s1);
+    }
+    __syncthreads();  // the buffer is refilled two chunks on
+  }
+  if (k <= rows) put_grad(p, s0, grad, a, q0, c1, c2);
+  if (k + 1 <= rows) put_grad(p + NH, s1, grad, a, q1, c1, c2);
 }
 
 __global__ void k_to_bf16(const float* theta, __nv_bfloat16* Wb) {
@@ -164,7 +296,6 @@ struct tc_mlp {
   float* theta = nullptr;  // FP32 master parameters
   float* m = nullptr;
   float* v = nullptr;
-  float* grad = nullptr;
   __nv_bfloat16* Wb = nullptr;  // BF16 copy (biases too, unused)
   float* norm = nullptr;        // x mean[36], x std[36], t mean[2], t std[2]
   float* work = nullptr;        // activations for up to kMaxB samples
@@ -174,7 +305,7 @@ struct tc_mlp {
 
 namespace {
 constexpr int kMaxB = 1024;
-constexpr size_t kWork = (size_t)kMaxB * (4 * NH + 2 * NO + NH * 2 + 1);
+constexpr size_t kWork = (size_t)kMaxB * (4 * NH + NO + 1);
 }  // namespace
 
 extern "C" int tc_mlp_create(tc_mlp** out, unsigned long long seed, tc_stream_t stream) {
@@ -185,7 +316,6 @@ extern "C" int tc_mlp_create(tc_mlp** out, unsigned long long seed, tc_stream_t 
   bool ok = cudaMalloc(&m->theta, MLP_NPARAMS * 4) == cudaSuccess &&
             cudaMalloc(&m->m, MLP_NPARAMS * 4) == cudaSuccess &&
             cudaMalloc(&m->v, MLP_NPARAMS * 4) == cudaSuccess &&
-            cudaMalloc(&m->grad, MLP_NPARAMS * 4) == cudaSuccess &&
             cudaMalloc(&m->Wb, MLP_NPARAMS * 2) == cudaSuccess &&
             cudaMalloc(&m->norm, MLP_NORM * 4) == cudaSuccess &&
             cudaMalloc(&m->work, kWork * 4) == cudaSuccess &&
@@ -210,7 +340,7 @@ extern "C" int tc_mlp_create(tc_mlp** out, unsigned long long seed, tc_stream_t 
 
 extern "C" int tc_mlp_destroy(tc_mlp* m) {
   if (!m) return TC_EINVAL;
-  void* ps[] = {m->theta, m->m, m->v, m->grad, m->Wb, m->norm, m->work, m->loss};
+  void* ps[] = {m->theta, m->m, m->v, m->Wb, m->norm, m->work, m->loss};
   for (void* p : ps)
     if (p) cudaFree(p);
   delete m;
@@ -242,38 +372,51 @@ extern "C" int tc_mlp_get_params(tc_mlp* m, float* theta, float* norm, tc_stream
 }
 
 namespace {
+// early: a launch that may start while its predecessor, a launch of the same
+// training call, finishes (the kernels wait in pdl_wait before they read or
+// write what it touches). The call's first launch starts in stream order: it
+// reads the caller's data before that wait.
+template <class... P, class... A>
+int launch_pdl(bool early, void (*kernel)(P...), int grid, int block, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = early ? 1 : 0;
+  TC_CUDA(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
+  return TC_OK;
+}
+
+// Loss and gradients of one batch, and with `a.theta` the Adam step on them.
 int fwd_bwd(tc_mlp* m, const float* X, const float* T, int B, float* grad, float* loss,
-            cudaStream_t st) {
-  float* Z1 = m->work;
-  float* H1 = Z1 + (size_t)kMaxB * NH;
-  float* Z2 = H1 + (size_t)kMaxB * NH;
-  float* H2 = Z2 + (size_t)kMaxB * NH;
-  float* OUT = H2 + (size_t)kMaxB * NH;
-  float* D = OUT + (size_t)kMaxB * NO;
+            const Adam& a, bool first, cudaStream_t st) {
+  float* H1 = m->work;
+  float* H2 = H1 + (size_t)kMaxB * NH;
+  float* D = H2 + (size_t)kMaxB * NH;
   float* dZ1 = D + (size_t)kMaxB * NO;
   float* dZ2 = dZ1 + (size_t)kMaxB * NH;
   float* lossb = dZ2 + (size_t)kMaxB * NH;
-  k_mlp_fwd<<<B, NH, 0, st>>>(X, B, m->Wb, m->theta, Z1, H1, Z2, H2, OUT);
-  k_mlp_bwd_act<<<B, NH, 0, st>>>(T, B, m->Wb, Z1, Z2, OUT, D, dZ1, dZ2, lossb);
-  k_mlp_bwd_w<<<(MLP_NPARAMS + 255) / 256, 256, 0, st>>>(X, B, H1, H2, D, dZ1, dZ2, lossb, grad,
-                                                         loss);
-  TC_CUDA(cudaGetLastError());
-  return TC_OK;
+  TC_TRY(launch_pdl(!first, k_mlp_samples, (B + SPC - 1) / SPC, SPC * NH, st, X, T, B, m->Wb, m->theta, H1,
+                    H2, (float*)nullptr, D, dZ1, dZ2, lossb));
+  return launch_pdl(true, k_mlp_grad, GCTAS, GT, st, X, B, H1, H2, D, dZ1, dZ2, lossb, grad, loss, a);
 }
 }  // namespace
 
 extern "C" int tc_mlp_loss_grad(tc_mlp* m, const float* X, const float* T, int B, float* loss,
                                 float* grad, tc_stream_t stream) {
   if (!m || !X || !T || !grad || B < 1 || B > kMaxB) return TC_EINVAL;
-  return fwd_bwd(m, X, T, B, grad, loss, (cudaStream_t)stream);
+  return fwd_bwd(m, X, T, B, grad, loss, Adam{}, true, (cudaStream_t)stream);
 }
 
 extern "C" int tc_mlp_forward(tc_mlp* m, const float* X, int B, float* Y, tc_stream_t stream) {
   if (!m || !X || !Y || B < 1) return TC_EINVAL;
-  k_mlp_fwd<<<B, NH, 0, (cudaStream_t)stream>>>(X, B, m->Wb, m->theta, nullptr, nullptr, nullptr,
-                                                nullptr, Y);
-  TC_CUDA(cudaGetLastError());
-  return TC_OK;
+  float* none = nullptr;
+  return launch_pdl(false, k_mlp_samples, (B + SPC - 1) / SPC, SPC * NH, (cudaStream_t)stream, X,
+                    none, B, m->Wb, m->theta, none, none, Y, none, none, none, none);
 }
 
 extern "C" int tc_mlp_train(tc_mlp* m, const float* X, const float* T, int N, int batch, int steps,
@@ -284,12 +427,10 @@ extern "C" int tc_mlp_train(tc_mlp* m, const float* X, const float* T, int N, in
   int off = 0;
   for (int s = 0; s < steps; ++s) {
     const int B = (off + batch <= N) ? batch : N - off;
-    TC_TRY(fwd_bwd(m, X + (size_t)off * MLP_IN, T + (size_t)off * MLP_OUT, B, m->grad,
-                   loss_hist ? loss_hist + s : m->loss, st));
     ++m->step;
-    k_adam<<<(MLP_NPARAMS + 255) / 256, 256, 0, st>>>(m->theta, m->grad, m->m, m->v, m->step, lr,
-                                                      m->Wb);
-    TC_CUDA(cudaGetLastError());
+    TC_TRY(fwd_bwd(m, X + (size_t)off * MLP_IN, T + (size_t)off * MLP_OUT, B, nullptr,
+                   loss_hist ? loss_hist + s : m->loss,
+                   Adam{m->theta, m->m, m->v, m->Wb, m->step, lr}, s == 0, st));
     off += B;
     if (off >= N) off = 0;
   }
