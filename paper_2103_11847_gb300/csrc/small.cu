@@ -10,66 +10,113 @@
 //      index on ties);
 //   3. y from the normal equations (H^T H + lambda^2 I) y = beta H^T e_1 by
 //      Cholesky.
-// GB300 runs FP64 at a small fraction of its FP32 rate, so everything here is
-// O(k^2)..O(k^3) work on k <= TC_MAX_PROJ numbers.
+//
+// Bound: FP64. GB300 issues fewer than two FP64 lanes a clock and SM, so a warp
+// instruction holds the pipe for about 19 clocks, and every division or square
+// root is a chain of them. So:
+// * a cluster of eight CTAs: rank 0 runs the SVD and the solve, and every rank
+//   evaluates 25 of a level's 200 grid points, one a lane of one warp (on one SM a
+//   level of k = 10 took about 35 us, nearly all of it the pipe);
+// * reciprocals and square roots by Newton's method (rcp_newton, rsqrt_newton:
+//   a few ulp), one reciprocal a GCV term;
+// * as many warps as the SVD has column pairs (at most 32), as every round ends
+//   in a barrier; the triangular solves run by columns over all threads.
+// At k = 10: 308 -> 176 us a launch (cold), most of it the SVD's chains.
+#include <cooperative_groups.h>
+
 #include "tc_device.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace {
 
-constexpr int NT = 1024;
-constexpr int NW = NT / 32;
 constexpr int NGRID = 200;
 constexpr int NLEVEL = 3;
 constexpr int MAX_SWEEPS = 40;
+constexpr int CL = 8;            // CTAs of the cluster
+constexpr int PPR = NGRID / CL;  // grid points a rank: one a lane
+static_assert(NGRID % CL == 0 && PPR <= 32, "one warp a rank");
 
-__device__ double gcv_eval(const double* sig, const double* g, int k, double gnull2,
-                           double lam, int variant) {
+// The hardware's estimates of 1 / sqrt(x) and 1 / x (about 20 bits; subnormals
+// as zero, zero gives Inf).
+__device__ __forceinline__ double rsqrt_approx(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  return y;
+}
+__device__ __forceinline__ double rcp_approx(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  return y;
+}
+
+// Lanes a column pair of the SVD: columns of up to 8 or 16 values share a warp.
+__host__ __device__ constexpr int lane_group(int rows) { return rows <= 8 ? 8 : rows <= 16 ? 16 : 32; }
+
+// GCV(lambda); sig2: squared singular values.
+__device__ double gcv_eval(const double* sig2, const double* g, int k, double gnull2, double lam,
+                           int variant) {
   const double l2 = lam * lam;
+  const double sc = variant == TC_GCV_FULL ? l2 : 1.0;
   double num = 0.0, den = 0.0;
+#pragma unroll 4
+  for (int i = 0; i < k; ++i) {
+    const double q = sc * rcp_newton(sig2[i] + l2);
+    const double r = g[i] * q;
+    num = fma(r, r, num);
+    den += q;
+  }
   if (variant == TC_GCV_FULL) {
-    for (int i = 0; i < k; ++i) {
-      const double d = sig[i] * sig[i] + l2;
-      const double r = l2 * g[i] / d;
-      num += r * r;
-      den += l2 / d;
-    }
     num += gnull2;
     den += 1.0;
-    return num / (den * den);
-  }
-  for (int i = 0; i < k; ++i) {
-    const double d = sig[i] * sig[i] + l2;
-    const double r = g[i] / d;
-    num += r * r;
-    den += 1.0 / d;
   }
   return num / (den * den);
 }
 
-__device__ double warp_sum_d(double v) {
+// First index of the smallest of v[0..n) over one warp (ties to the lower index).
+__device__ int warp_argmin(const double* v, int n) {
+  double best = INFINITY;
+  int bi = n;
+  for (int t = threadIdx.x & 31; t < n; t += 32)
+    if (v[t] < best) {
+      best = v[t];
+      bi = t;
+    }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+  for (int o = 16; o > 0; o >>= 1) {
+    const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+    if (ob < best || (ob == best && oi < bi)) {
+      best = ob;
+      bi = oi;
+    }
+  }
+  return bi < n ? bi : 0;
 }
 
 // Dynamic shared memory: Hs[(k+1) * kk] (column-major working copy, kk = k
 // rounded up to even), reused as the k x k normal matrix afterwards.
-__global__ void __launch_bounds__(NT)
+__global__ void __launch_bounds__(1024)
 k_tikhonov_gcv(const double* __restrict__ H, int ld, int kmax, const int* kdev,
                const double* beta_p, int variant, double lambda_in, double* lambda_out,
                double* y, double* gcv_out, const int* skip) {
-  if (skip && *skip) return;
+  if (skip && *skip) return;  // uniform over the cluster, as is every return below
   extern __shared__ double dsm[];
-  __shared__ double sig[TC_MAX_PROJ], g[TC_MAX_PROJ], dn[TC_MAX_PROJ];
-  __shared__ double vals[NGRID];
-  __shared__ double grid[NGRID];
+  __shared__ double sig2[TC_MAX_PROJ], g[TC_MAX_PROJ], dn[TC_MAX_PROJ];
+  __shared__ double vals[NGRID], grid[NGRID];
+  __shared__ double bracket[NLEVEL + 1][2], sh_w[32];
+  __shared__ double sh_gnull2, sh_lam, sh_gcv;
+  __shared__ double rot[TC_MAX_PROJ / 2][2];  // a pair's dot product, then its c and s
   __shared__ int sh_rot;
-  __shared__ double sh_misc[8];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nt = blockDim.x, nw = nt / 32;
   const int k = kdev ? min(*kdev, kmax) : kmax;
   const double beta = *beta_p;
+  const bool search = !(lambda_in >= 0.0);
   if (k <= 0) {
-    if (tid == 0) {
+    if (rank == 0 && tid == 0) {
       *lambda_out = nan("");
       if (gcv_out) *gcv_out = nan("");
     }
@@ -77,170 +124,229 @@ k_tikhonov_gcv(const double* __restrict__ H, int ld, int kmax, const int* kdev,
   }
   const int rows = k + 1;
   const int kk = k + (k & 1);
-  double* Hs = dsm;  // column c at Hs + c*rows
-  for (int idx = tid; idx < rows * kk; idx += NT) {
-    const int c = idx / rows, r = idx % rows;
-    Hs[idx] = (c < k) ? H[(size_t)r * ld + c] : 0.0;
-  }
-  __syncthreads();
-
-  // ---- 1. one-sided Jacobi -------------------------------------------------
-  // Rotate while |<h_p, h_q>| > rows * eps * ||h_p|| ||h_q||: below that the
-  // inner product is rounding noise of the (rows)-term dot product. Each warp
-  // rotates one column pair of the round; squared column norms d[] are
-  // recomputed every sweep and updated by the exact rotation identities
-  // d_p -= t gamma, d_q += t gamma in between.
-  const double jtol = rows * 2.220446049250313e-16;
-  const int npairs = kk / 2;
-  for (int sweep = 0; sweep < MAX_SWEEPS; ++sweep) {
-    if (tid == 0) sh_rot = 0;
-    for (int c = warp; c < kk; c += NW) {
-      const double* x = Hs + (size_t)c * rows;
-      double s2 = 0.0;
-      for (int r = lane; r < rows; r += 32) s2 += x[r] * x[r];
-      s2 = warp_sum_d(s2);
-      if (lane == 0) dn[c] = s2;
+  if (rank == 0) {
+    double* Hs = dsm;  // column c at Hs + c*rows
+    for (int idx = tid; idx < rows * kk; idx += nt) {
+      const int c = idx / rows, r = idx % rows;
+      Hs[idx] = (c < k) ? H[(size_t)r * ld + c] : 0.0;
     }
     __syncthreads();
-    for (int rnd = 0; rnd < kk - 1; ++rnd) {
-      for (int pi = warp; pi < npairs; pi += NW) {
-        // circle method: player 0 fixed, the others rotate by rnd
-        const int a = (pi == 0) ? 0 : ((pi - 1 + rnd) % (kk - 1)) + 1;
-        const int b = ((kk - 2 - pi + rnd) % (kk - 1)) + 1;
-        double* xp = Hs + (size_t)a * rows;
-        double* xq = Hs + (size_t)b * rows;
-        double ga = 0.0;
-        for (int r = lane; r < rows; r += 32) ga += xp[r] * xq[r];
-        ga = warp_sum_d(ga);
-        const double al = dn[a], be = dn[b];
-        if (ga != 0.0 && fabs(ga) > jtol * sqrt(al * be)) {
-          const double zeta = (be - al) / (2.0 * ga);
-          const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-          const double c = 1.0 / sqrt(1.0 + t * t);
-          const double s = c * t;
-          for (int r = lane; r < rows; r += 32) {
-            const double u = xp[r], v = xq[r];
-            xp[r] = c * u - s * v;
-            xq[r] = s * u + c * v;
-          }
-          if (lane == 0) {
+
+    // ---- 1. one-sided Jacobi -----------------------------------------------
+    // Rotate while |<h_p, h_q>| > rows * eps * ||h_p|| ||h_q||: below that the
+    // inner product is rounding noise of the (rows)-term dot product. Squared
+    // column norms d[] are recomputed every sweep and updated by the rotation
+    // identities d_p -= t gamma, d_q += t gamma in between. A round is three
+    // parts: the pairs' dot products (LG lanes a pair), their rotations (one
+    // lane a pair, so that the FP64 chains of all pairs share a warp's
+    // instructions), and the column updates. t comes from a 20-bit estimate: the
+    // rotation is orthogonal to FP64 (c and s = c t belong to that t), and it
+    // leaves 1e-6 of gamma where the exact t would leave nothing, which the next
+    // sweep's quadratic convergence hides.
+    const double jtol = rows * 2.220446049250313e-16;
+    const int npairs = kk / 2, lg = lane_group(rows), ppw = 32 / lg, sub = lane % lg;
+    auto pair_of = [&](int pi, int rnd, int& a, int& b) {
+      // circle method: player 0 fixed, the others rotate by rnd
+      a = (pi == 0) ? 0 : ((pi - 1 + rnd) % (kk - 1)) + 1;
+      b = ((kk - 2 - pi + rnd) % (kk - 1)) + 1;
+    };
+    for (int sweep = 0; sweep < MAX_SWEEPS; ++sweep) {
+      if (tid == 0) sh_rot = 0;
+      for (int c = warp; c < kk; c += nw) {
+        const double* x = Hs + (size_t)c * rows;
+        double s2 = 0.0;
+        for (int r = lane; r < rows; r += 32) s2 += x[r] * x[r];
+        s2 = warp_sum(s2);
+        if (lane == 0) dn[c] = s2;
+      }
+      for (int rnd = 0; rnd < kk - 1; ++rnd) {
+        for (int p0 = warp * ppw; p0 < npairs; p0 += nw * ppw) {
+          const int pi = p0 + lane / lg;
+          int a, b;
+          pair_of(min(pi, npairs - 1), rnd, a, b);
+          double ga = 0.0;
+          for (int r = sub; r < rows; r += lg) ga = fma(Hs[a * rows + r], Hs[b * rows + r], ga);
+          for (int o = lg / 2; o > 0; o >>= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
+          if (sub == 0 && pi < npairs) rot[pi][0] = ga;
+        }
+        __syncthreads();
+        if (tid < npairs) {
+          int a, b;
+          pair_of(tid, rnd, a, b);
+          const double ga = rot[tid][0], al = dn[a], be = dn[b];
+          double c = 1.0, sn = 0.0;
+          if (ga != 0.0 && fabs(ga) * rsqrt_approx(al * be) > jtol) {
+            const float z = (float)((be - al) * rcp_approx(2.0 * ga));
+            const float az = fabsf(z);
+            // 1 / (|z| + sqrt(1 + z^2)), past FP32's range of z^2 1 / (2 |z|)
+            const float ta = az < 1e18f ? 1.f / (az + sqrtf(fmaf(z, z, 1.f))) : 0.5f / az;
+            const double t = z >= 0.f ? ta : -ta;
+            c = rsqrt_approx(fma(t, t, 1.0));
+            sn = c * t;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {  // to c^2 + s^2 = 1 within an ulp: hundreds of
+              const double e = fma(-sn, sn, fma(-c, c, 1.0));  // rotations meet in a column
+              c = fma(0.5 * c, e, c);
+              sn = fma(0.5 * sn, e, sn);
+            }
             dn[a] = al - t * ga;
             dn[b] = be + t * ga;
             sh_rot = 1;
           }
+          rot[tid][0] = c;
+          rot[tid][1] = sn;
         }
+        __syncthreads();
+        for (int p0 = warp * ppw; p0 < npairs; p0 += nw * ppw) {
+          const int pi = p0 + lane / lg;
+          if (pi >= npairs) continue;
+          const double c = rot[pi][0], sn = rot[pi][1];
+          if (sn == 0.0) continue;
+          int a, b;
+          pair_of(pi, rnd, a, b);
+          for (int r = sub; r < rows; r += lg) {
+            const double u = Hs[a * rows + r], v = Hs[b * rows + r];
+            Hs[a * rows + r] = c * u - sn * v;
+            Hs[b * rows + r] = sn * u + c * v;
+          }
+        }
+        __syncthreads();
       }
+      const int any = sh_rot;
       __syncthreads();
+      if (!any) break;
     }
-    const int any = sh_rot;
-    __syncthreads();
-    if (!any) break;
-  }
-  for (int c = warp; c < k; c += NW) {
-    const double* x = Hs + (size_t)c * rows;
-    double s2 = 0.0;
-    for (int r = lane; r < rows; r += 32) s2 += x[r] * x[r];
-    s2 = warp_sum_d(s2);
-    if (lane == 0) {
-      const double sv = sqrt(s2);
-      sig[c] = sv;
-      g[c] = (sv > 0.0) ? beta * x[0] / sv : 0.0;
+    for (int c = warp; c < k; c += nw) {
+      const double* x = Hs + (size_t)c * rows;
+      double s2 = 0.0;
+      for (int r = lane; r < rows; r += 32) s2 += x[r] * x[r];
+      s2 = warp_sum(s2);
+      if (lane == 0) {
+        sig2[c] = s2;
+        g[c] = (s2 > 0.0) ? beta * x[0] * (1.0 / sqrt(s2)) : 0.0;
+      }
     }
-  }
-  __syncthreads();
-  if (tid == 0) {  // the part of beta e1 outside the range of H
-    double gs = 0.0;
-    for (int i = 0; i < k; ++i) gs += g[i] * g[i];
-    sh_misc[2] = fmax(beta * beta - gs, 0.0);
-  }
-  __syncthreads();
-  const double gnull2 = sh_misc[2];
-
-  // ---- 2. lambda -------------------------------------------------------------
-  double lam = lambda_in;
-  if (!(lambda_in >= 0.0)) {
     double hs = 0.0;  // ||H||_F
-    for (int idx = tid; idx < rows * k; idx += NT) {
+    for (int idx = tid; idx < rows * k; idx += nt) {
       const double v = H[(size_t)(idx / k) * ld + idx % k];
       hs += v * v;
     }
-    hs = warp_sum_d(hs);
-    if (lane == 0) vals[warp] = hs;
+    hs = warp_sum(hs);
+    if (lane == 0) sh_w[warp] = hs;
     __syncthreads();
-    if (tid == 0) {
-      double t = 0.0;
-      for (int w = 0; w < NW; ++w) t += vals[w];
-      sh_misc[5] = log(sqrt(t)) - 10.0 * log(10.0);
-      sh_misc[6] = log(sqrt(t));
+    if (warp == 0) {
+      const double t = warp_sum(lane < nw ? sh_w[lane] : 0.0);
+      double gs = 0.0;  // the part of beta e1 outside the range of H
+      for (int i = lane; i < k; i += 32) gs += g[i] * g[i];
+      gs = warp_sum(gs);
+      if (lane == 0) {
+        // below the rounding of the sum it is a difference of equal numbers: zero
+        const double d = beta * beta - gs;
+        sh_gnull2 = d > rows * 2.220446049250313e-16 * beta * beta ? d : 0.0;
+        bracket[0][1] = log(sqrt(t));
+        bracket[0][0] = bracket[0][1] - 10.0 * log(10.0);
+      }
     }
     __syncthreads();
-    for (int level = 0; level < NLEVEL; ++level) {
-      const double lo = sh_misc[5], hi = sh_misc[6];
-      const double step = (hi - lo) / (NGRID - 1);
-      for (int i = tid; i < NGRID; i += NT) {
-        grid[i] = exp(i == NGRID - 1 ? hi : lo + i * step);
-        vals[i] = gcv_eval(sig, g, k, gnull2, grid[i], variant);
-      }
-      __syncthreads();
-      if (tid == 0) {
-        int bi = 0;
-        for (int i = 1; i < NGRID; ++i)
-          if (vals[i] < vals[bi]) bi = i;
-        sh_misc[3] = grid[bi];
-        sh_misc[4] = vals[bi];
-        sh_misc[5] = log(grid[max(bi - 1, 0)]);
-        sh_misc[6] = log(grid[min(bi + 1, NGRID - 1)]);
-      }
-      __syncthreads();
-    }
-    lam = sh_misc[3];
-  } else if (tid == 0) {
-    sh_misc[4] = gcv_eval(sig, g, k, gnull2, lam, variant);
   }
+
+  // ---- 2. lambda -------------------------------------------------------------
+  if (search) {
+    cluster.sync();  // every CTA runs, and rank 0's values are in place
+    if (rank != 0) {
+      for (int i = tid; i < k; i += nt) {
+        sig2[i] = cluster.map_shared_rank(sig2, 0)[i];
+        g[i] = cluster.map_shared_rank(g, 0)[i];
+      }
+      if (tid == 0) {
+        sh_gnull2 = *cluster.map_shared_rank(&sh_gnull2, 0);
+        bracket[0][0] = cluster.map_shared_rank(&bracket[0][0], 0)[0];
+        bracket[0][1] = cluster.map_shared_rank(&bracket[0][0], 0)[1];
+      }
+      __syncthreads();
+    }
+    for (int level = 0; level < NLEVEL; ++level) {
+      if (warp == 0) {  // points PPR rank .. + PPR - 1
+        const double lo = bracket[level][0], hi = bracket[level][1];
+        const double step = (hi - lo) / (NGRID - 1);
+        const int i = rank * PPR + lane;
+        if (lane < PPR) {
+          const double lam = exp(i == NGRID - 1 ? hi : lo + i * step);
+          const double v = gcv_eval(sig2, g, k, sh_gnull2, lam, variant);
+          cluster.map_shared_rank(grid, 0)[i] = lam;
+          cluster.map_shared_rank(vals, 0)[i] = v;
+        }
+      }
+      cluster.sync();  // the level's values are in rank 0
+      if (rank == 0 && warp == 0) {
+        const int bi = warp_argmin(vals, NGRID);
+        if (lane == 0) {
+          sh_lam = grid[bi];
+          sh_gcv = vals[bi];
+        }
+        if (level + 1 < NLEVEL) {
+          const double e = lane < 2 ? log(grid[lane == 0 ? max(bi - 1, 0) : min(bi + 1, NGRID - 1)]) : 0.0;
+          const double lo = __shfl_sync(0xffffffffu, e, 0), hi = __shfl_sync(0xffffffffu, e, 1);
+          if (lane < CL) {
+            double* q = cluster.map_shared_rank(&bracket[0][0], lane) + 2 * (level + 1);
+            q[0] = lo;
+            q[1] = hi;
+          }
+        }
+      }
+      if (level + 1 < NLEVEL) cluster.sync();  // the next bracket is everywhere
+    }
+  } else if (rank == 0 && tid == 0) {
+    sh_lam = lambda_in;
+    sh_gcv = gcv_eval(sig2, g, k, sh_gnull2, lambda_in, variant);
+  }
+  if (rank != 0) return;  // no rank reads another's shared memory from here on
   __syncthreads();
+  const double lam = sh_lam;
   if (tid == 0) {
     *lambda_out = lam;
-    if (gcv_out) *gcv_out = sh_misc[4];
+    if (gcv_out) *gcv_out = sh_gcv;
   }
 
   // ---- 3. (H^T H + lambda^2 I) y = beta H^T e_1, Cholesky --------------------
-  double* G = dsm;  // k x k row-major, overwrites the Jacobi copy
-  __syncthreads();
-  for (int idx = tid; idx < k * k; idx += NT) {
+  double* G = dsm;  // k x k row-major, overwrites the Jacobi copy; L's diagonal
+  double* inv = dn;  // is kept inverted in dn
+  for (int idx = tid; idx < k * k; idx += nt) {
     const int i = idx / k, jj = idx % k;
     double s = 0.0;
     for (int r = 0; r < rows; ++r) s += H[(size_t)r * ld + i] * H[(size_t)r * ld + jj];
     if (i == jj) s += lam * lam;
     G[idx] = s;
   }
-  for (int i = tid; i < k; i += NT) g[i] = beta * H[i];  // rhs = beta * (row 1 of H)
+  for (int i = tid; i < k; i += nt) g[i] = beta * H[i];  // rhs = beta * (row 1 of H)
   __syncthreads();
   for (int c = 0; c < k; ++c) {
-    if (tid == 0) G[c * k + c] = sqrt(G[c * k + c]);
+    if (tid == 0) inv[c] = rsqrt_newton(G[c * k + c]);
     __syncthreads();
-    const double d = G[c * k + c];
-    for (int r = c + 1 + tid; r < k; r += NT) G[r * k + c] /= d;
+    const double d = inv[c];
+    for (int r = c + 1 + tid; r < k; r += nt) G[r * k + c] *= d;
     __syncthreads();
-    for (int idx = tid; idx < (k - c - 1) * (k - c - 1); idx += NT) {
+    for (int idx = tid; idx < (k - c - 1) * (k - c - 1); idx += nt) {
       const int r = c + 1 + idx / (k - c - 1), q = c + 1 + idx % (k - c - 1);
       if (q <= r) G[r * k + q] -= G[r * k + c] * G[q * k + c];
     }
     __syncthreads();
   }
-  if (tid == 0) {
-    for (int r = 0; r < k; ++r) {  // L z = rhs
-      double s = g[r];
-      for (int q = 0; q < r; ++q) s -= G[r * k + q] * sig[q];
-      sig[r] = s / G[r * k + r];
-    }
-    for (int r = k - 1; r >= 0; --r) {  // L^T y = z
-      double s = sig[r];
-      for (int q = r + 1; q < k; ++q) s -= G[q * k + r] * g[q];
-      g[r] = s / G[r * k + r];
-    }
+  for (int c = 0; c < k; ++c) {  // L z = rhs by columns: g[c] becomes z[c] / 1
+    const double z = g[c] * inv[c];
+    __syncthreads();
+    for (int r = c + 1 + tid; r < k; r += nt) g[r] -= G[r * k + c] * z;
+    if (tid == 0) g[c] = z;
+    __syncthreads();
   }
-  __syncthreads();
-  for (int i = tid; i < kmax; i += NT) y[i] = (i < k) ? g[i] : 0.0;
+  for (int c = k - 1; c >= 0; --c) {  // L^T y = z by columns of L^T
+    const double z = g[c] * inv[c];
+    __syncthreads();
+    for (int r = tid; r < c; r += nt) g[r] -= G[c * k + r] * z;
+    if (tid == 0) g[c] = z;
+    __syncthreads();
+  }
+  for (int i = tid; i < kmax; i += nt) y[i] = (i < k) ? g[i] : 0.0;
 }
 
 __global__ void k_build_bidiag(const double* alpha, const double* beta, const int* kdev,
@@ -268,9 +374,23 @@ int launch_tikhonov_gcv(const double* H, int ld, int kmax, const int* kdev,
   size_t smem = sizeof(double) * (size_t)(kmax + 1) * kk;
   const size_t gsz = sizeof(double) * (size_t)kmax * kmax;
   if (gsz > smem) smem = gsz;
-  k_tikhonov_gcv<<<1, NT, smem, st>>>(H, ld, kmax, kdev, beta, variant, lambda_in, lambda_out,
-                                      y, gcv_out, skip);
-  TC_CUDA(cudaGetLastError());
+  const int ppw = 32 / lane_group(kmax + 1);
+  int nw = (kk / 2 + ppw - 1) / ppw;  // the warps that the column pairs fill
+  nw = nw < 4 ? 4 : nw > 32 ? 32 : nw;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(CL);
+  cfg.blockDim = dim3(32 * nw);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = CL;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  TC_CUDA(cudaLaunchKernelEx(&cfg, k_tikhonov_gcv, H, ld, kmax, kdev, beta, variant, lambda_in,
+                             lambda_out, y, gcv_out, skip));
   return TC_OK;
 }
 

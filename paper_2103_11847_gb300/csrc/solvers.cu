@@ -554,6 +554,10 @@ extern "C" int tc_gmres_c(tc_plan* p, const float* C, const float* X0, float* X,
       ea.red = make_red(p, hcol, 0, Vb, flags + 2);
       ea.skip = flags + 4;
       TC_TRY(cprod_epi(p, Vj, Wn, ea, st));
+      if (arnoldi_step_fits(T)) {
+        TC_TRY(launch_arnoldi_step(Vb, T, hcol, m, j, flags, st));
+        continue;
+      }
       for (int i = 0; i <= j; ++i) {  // MGS: W -= h_ij V_i, then the next product
         const bool last = (i == j);
         Red r = make_red(p, H + (size_t)(i + 1) * m + j, last ? 1 : 0,

@@ -279,7 +279,14 @@ int launch_combine2(float* X, const double* y, float* X2, const double* y2, cons
                     cudaStream_t st);
 int launch_mgs_pass(float* W, const float* Vi, const double* h, const float* Vnext,
                     size_t n, const Red& red, const int* skip, cudaStream_t st);
-// small.cu (FP64, one CTA)
+// The rest of Algorithm 2's step j after its product (every pass, the
+// normalisation and the flags of k_gmres_step_done) in one launch, for tensors
+// that fit one cluster. V: the basis, n apart, W at V + (j + 1) n; Hcol: column j
+// of H, row stride ld, h_0j in place.
+bool arnoldi_step_fits(size_t n);
+int launch_arnoldi_step(float* V, size_t n, double* Hcol, int ld, int j, int* flags,
+                        cudaStream_t st);
+// small.cu (FP64)
 int launch_tikhonov_gcv(const double* H, int ld, int kmax, const int* kdev,
                         const double* beta, int variant, double lambda_in,
                         double* lambda_out, double* y, double* gcv_out, const int* skip,

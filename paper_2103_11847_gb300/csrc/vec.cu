@@ -2,6 +2,8 @@
 // products (Definition 2.2), scaled copies, the LSQR update of Algorithm 6
 // steps (c)-(g), the basis combination V (*) y (§3.1, eq. (xm)), and one
 // modified Gram-Schmidt pass of Algorithm 2 fused with the next inner product.
+#include <cooperative_groups.h>
+
 #include "tc_device.cuh"
 
 namespace {
@@ -21,15 +23,23 @@ k_reduce(const float* __restrict__ x, const float* __restrict__ other, size_t n,
   if (skip && *skip) return;
   float s = 0.f;
   const size_t stride = (size_t)gridDim.x * NT;
-  for (size_t i = (size_t)blockIdx.x * NT + threadIdx.x; i < n; i += stride) {
-    const float v = x[i];
-    s = fmaf(v, other ? other[i] : v, s);
+  for (size_t i0 = (size_t)blockIdx.x * NT + threadIdx.x; i0 < n; i0 += 8 * stride) {
+    float v[8], o[8];  // eight loads in flight a thread
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const size_t i = i0 + u * stride;
+      v[u] = i < n ? x[i] : 0.f;
+      o[u] = other && i < n ? other[i] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (i0 + u * stride < n) s = fmaf(v[u], other ? o[u] : v[u], s);
   }
   reduce_finish(s, red);
 }
 
 __global__ void __launch_bounds__(NT)
-k_scale(const float* __restrict__ in, float* out, size_t n, Coef c, const float* prev,
+k_scale(const float* in, float* out, size_t n, Coef c, const float* prev,
         const int* skip) {
   if (skip && *skip) return;
   __shared__ float sh[2];
@@ -37,10 +47,22 @@ k_scale(const float* __restrict__ in, float* out, size_t n, Coef c, const float*
   __syncthreads();
   const float ca = sh[0], cp = sh[1];
   const size_t stride = (size_t)gridDim.x * NT;
-  for (size_t i = (size_t)blockIdx.x * NT + threadIdx.x; i < n; i += stride) {
-    float o = ca * in[i];
-    if (prev) o = fmaf(cp, prev[i], o);
-    out[i] = o;
+  for (size_t i0 = (size_t)blockIdx.x * NT + threadIdx.x; i0 < n; i0 += 8 * stride) {
+    float v[8], p[8];  // eight loads in flight a thread (out may alias in or prev)
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const size_t i = i0 + u * stride;
+      v[u] = i < n ? in[i] : 0.f;
+      p[u] = prev && i < n ? prev[i] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const size_t i = i0 + u * stride;
+      if (i >= n) break;
+      float o = ca * v[u];
+      if (prev) o = fmaf(cp, p[u], o);
+      out[i] = o;
+    }
   }
 }
 
@@ -310,7 +332,9 @@ k_epi(const float* __restrict__ in, float* out, size_t n, Epi ep, int vec) {
   if (ep.red.out) reduce_finish(local, ep.red);
 }
 
-// Algorithm 2 step 3(b): W -= h V_i, then <V_next, W> (or ||W||^2) for the next step.
+// Algorithm 2 step 3(b): W -= h V_i, then <V_next, W> (or ||W||^2) for the next
+// step. Eight elements' loads are in flight before the first store (W may not
+// be known not to alias the basis, so the compiler keeps loads behind stores).
 __global__ void __launch_bounds__(NT)
 k_mgs_pass(float* W, const float* __restrict__ Vi, const double* h, const float* Vnext,
            size_t n, Red red, const int* skip) {
@@ -321,12 +345,169 @@ k_mgs_pass(float* W, const float* __restrict__ Vi, const double* h, const float*
   const float hh = sh_h;
   float s = 0.f;
   const size_t st = (size_t)gridDim.x * NT;
-  for (size_t i = (size_t)blockIdx.x * NT + threadIdx.x; i < n; i += st) {
-    const float w = fmaf(-hh, Vi[i], W[i]);
-    W[i] = w;
-    s = fmaf(w, Vnext ? Vnext[i] : w, s);
+  for (size_t i0 = (size_t)blockIdx.x * NT + threadIdx.x; i0 < n; i0 += 8 * st) {
+    float w[8], v[8], x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const size_t i = i0 + u * st;
+      w[u] = i < n ? W[i] : 0.f;
+      v[u] = i < n ? Vi[i] : 0.f;
+      x[u] = Vnext && i < n ? Vnext[i] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const size_t i = i0 + u * st;
+      if (i >= n) break;
+      w[u] = fmaf(-hh, v[u], w[u]);
+      W[i] = w[u];
+      s = fmaf(w[u], Vnext ? x[u] : w[u], s);
+    }
   }
   reduce_finish(s, red);
+}
+
+// Step j of Algorithm 2 after its product, in one launch: for i = 0 .. j, W -=
+// h_ij V_i and h_{i+1,j} = <V_{i+1}, W> (at i = j ||W||), then V_{j+1} = W /
+// h_{j+1,j} and the step's flags (as k_gmres_step_done). h_0j is in place.
+//
+// Bound: latency, j + 1 dependent reductions over the tensor. As a launch a pass
+// (48 CTAs, W through HBM) a 256 x 256 x 3 pass took about 13 us; here a tensor
+// of up to 64 CTAs' worth of elements (n <= 262144) stays in the registers of
+// one thread-block cluster of 16 CTAs, the next V_i is loaded while a
+// reduction runs, and a reduction is the CTAs' partial sums pushed into every
+// CTA's shared memory, one cluster barrier, and the sum taken by every CTA: 55
+// passes in about 0.1 ms. A larger tensor takes the separate launches: one
+// cluster's 16 SMs would be short of bandwidth and registers.
+// The element order and the reduction tree are the separate launches' (NV =
+// grid_for(n, 16) virtual CTAs of 256 threads, VC of them a CTA), so the bits
+// are the same.
+constexpr int AO_CL = 16, AO_E = 16;  // CTAs of the cluster, elements a thread
+
+struct ArnoldiStep {
+  float* V;        // the basis, n apart: V_0 .. V_j, and W in place of V_{j+1}
+  size_t n;
+  double* H;       // column j: H(i, j) at H[i * ld]
+  int ld, j, nv;
+  int* flags;      // [1] steps [2] status [3] steps of the cycle [4] stop
+};
+
+template <int VC>
+__global__ void __launch_bounds__(VC * NT, 1) k_arnoldi_step(ArnoldiStep a) {
+  if (a.flags[4]) return;  // uniform over the cluster
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  __shared__ float sh_w[VC][8];
+  __shared__ double sh_h;
+  __shared__ double sh_p[2][64];  // the virtual CTAs' partials, by pass parity
+  const int tid = threadIdx.x, lane = tid & 31, vc = tid / NT;
+  const int v = (int)cluster.block_rank() * VC + vc;  // virtual CTA
+  const size_t st = (size_t)a.nv * NT, i0 = (size_t)v * NT + tid % NT;
+  float* W = a.V + (size_t)(a.j + 1) * a.n;
+  float w[AO_E], x[AO_E], y[AO_E];
+  auto load = [&](const float* src, float (&r)[AO_E]) {
+#pragma unroll
+    for (int u = 0; u < AO_E; ++u) {
+      const size_t i = i0 + u * st;
+      r[u] = v < a.nv && i < a.n ? src[i] : 0.f;
+    }
+  };
+  load(W, w);
+  load(a.V, x);
+  if (a.j > 0) load(a.V + a.n, y);
+  if (tid < 128) sh_p[tid >> 6][tid & 63] = 0.0;
+  cluster.sync();  // every CTA's partials are cleared before a peer writes one
+  double h = a.H[0];
+  for (int i = 0; i <= a.j; ++i) {
+    const bool last = i == a.j;
+    const float hh = (float)h;
+    float s = 0.f;
+#pragma unroll
+    for (int u = 0; u < AO_E; ++u) {
+      if (v < a.nv && i0 + u * st < a.n) {
+        w[u] = fmaf(-hh, x[u], w[u]);
+        s = fmaf(w[u], last ? w[u] : y[u], s);
+      }
+      x[u] = y[u];
+    }
+    if (i + 2 <= a.j) load(a.V + (size_t)(i + 2) * a.n, y);
+    s = warp_sum_f(s);
+    if (lane == 0) sh_w[vc][(tid % NT) >> 5] = s;
+    __syncthreads();
+    double* part = sh_p[i & 1];
+    if (tid < 32 * VC) {  // warp q: virtual CTA q of this CTA; lane r: to rank r
+      const int q = tid >> 5, qv = (int)cluster.block_rank() * VC + q;
+      float wf = lane < 8 ? sh_w[q][lane] : 0.f;
+      wf = warp_sum_f(wf);
+      if (lane < AO_CL && qv < a.nv) cluster.map_shared_rank(part, lane)[qv] = (double)wf;
+    }
+    cluster.sync();
+    if (tid < 32) {  // one warp a CTA: FP64 is scarce
+      // the sum in the order of a 256-thread CTA: threads 0 .. 31, 32 .. 63, the two
+      const double total = warp_sum(part[lane]) + warp_sum(part[32 + lane]);
+      const double r = last ? sqrt(total) : total;
+      if (lane == 0) {
+        sh_h = r;
+        if (cluster.block_rank() == 0) {
+          if (!isfinite(total)) a.flags[2] = TC_ENONFINITE;
+          a.H[(size_t)(i + 1) * a.ld] = r;
+        }
+      }
+    }
+    __syncthreads();
+    h = sh_h;
+  }
+  __shared__ float sh_ca;
+  if (tid == 0) sh_ca = (h != 0.0) ? (float)rcp_newton(h) : 0.f;
+  __syncthreads();
+  const float ca = sh_ca;
+#pragma unroll
+  for (int u = 0; u < AO_E; ++u)
+    if (v < a.nv && i0 + u * st < a.n) W[i0 + u * st] = ca * w[u];
+  if (cluster.block_rank() == 0 && tid == 0) {
+    a.flags[3] = a.j + 1;
+    a.flags[1] += 1;
+    if (!(h > 0.0)) a.flags[4] = 1;  // h_{j+1,j} = 0 (or NaN): stop this cycle
+  }
+}
+
+template <int VC>
+int launch_ao(const ArnoldiStep& a, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(AO_CL);
+  cfg.blockDim = dim3(VC * NT);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = AO_CL;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  TC_CUDA(cudaLaunchKernelEx(&cfg, k_arnoldi_step<VC>, a));
+  return TC_OK;
+}
+
+bool g_ao_ok = false;  // the device runs such a cluster (set by vec_init)
+
+// Clusters of 16 are past the portable size: ask for them, and see that one fits.
+template <int VC>
+int init_ao(bool* ok) {
+  TC_CUDA(cudaFuncSetAttribute(k_arnoldi_step<VC>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(AO_CL);
+  cfg.blockDim = dim3(VC * NT);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = AO_CL;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, k_arnoldi_step<VC>, &cfg);
+  if (e != cudaSuccess) cudaGetLastError();
+  if (e != cudaSuccess || n < 1) *ok = false;
+  return TC_OK;
 }
 
 }  // namespace
@@ -340,6 +521,11 @@ int vec_init() {
   TC_CUDA(cudaFuncSetAttribute(k_scale, cudaFuncAttributePreferredSharedMemoryCarveout, c));
   TC_CUDA(cudaFuncSetAttribute(k_lsqr_update<float>, cudaFuncAttributePreferredSharedMemoryCarveout, c));
   TC_CUDA(cudaFuncSetAttribute(k_lsqr_update<float4>, cudaFuncAttributePreferredSharedMemoryCarveout, c));
+  g_ao_ok = true;
+  TC_TRY(init_ao<1>(&g_ao_ok));
+  TC_TRY(init_ao<2>(&g_ao_ok));
+  TC_TRY(init_ao<3>(&g_ao_ok));
+  TC_TRY(init_ao<4>(&g_ao_ok));
   int dev = 0;
   TC_CUDA(cudaGetDevice(&dev));
   TC_CUDA(cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev));
@@ -454,6 +640,21 @@ int launch_mgs_pass(float* W, const float* Vi, const double* h, const float* Vne
   k_mgs_pass<<<grid_for(n, 16), NT, 0, st>>>(W, Vi, h, Vnext, n, red, skip);
   TC_CUDA(cudaGetLastError());
   return TC_OK;
+}
+
+bool arnoldi_step_fits(size_t n) { return g_ao_ok && grid_for(n, AO_E) <= 4 * AO_CL; }
+
+int launch_arnoldi_step(float* V, size_t n, double* Hcol, int ld, int j, int* flags,
+                        cudaStream_t st) {
+  TC_CHECK(arnoldi_step_fits(n) && j >= 0);
+  const int nv = (int)grid_for(n, AO_E);
+  const ArnoldiStep a{V, n, Hcol, ld, j, nv, flags};
+  switch ((nv + AO_CL - 1) / AO_CL) {
+    case 1: return launch_ao<1>(a, st);
+    case 2: return launch_ao<2>(a, st);
+    case 3: return launch_ao<3>(a, st);
+    default: return launch_ao<4>(a, st);
+  }
 }
 
 namespace {
