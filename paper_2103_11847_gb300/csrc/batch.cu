@@ -94,7 +94,7 @@ extern "C" int tc_lsqr_c_batched(tc_batch* b, const float* const* C, float* cons
     cudaStream_t st = (cudaStream_t)stream;
     TC_TRY(group_prepare(&b->grp, b->plans, C, X, X_reg, itermax, st));
     if (b->batch_mode == 0) TC_TRY(group_autotune(&b->grp, b->plans[0], st));
-    else TC_TRY(group_fix_tile(&b->grp, b->batch_mode - 2, st));
+    else TC_TRY(group_fix_tile(&b->grp, b->batch_mode - 2));
     cudaGraph_t g = nullptr;
     TC_CUDA(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
     const int rc = group_enqueue(&b->grp, b->plans[0], tol, lambda, infos, b->cap);

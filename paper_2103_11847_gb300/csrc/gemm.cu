@@ -157,10 +157,11 @@ struct Out {
   float ca, cp;
 };
 
+template <bool EPI>  // a product's last stage (EPI) is never stored transposed
 __device__ __forceinline__ void out_one(const Out& o, int l, int row, int col, float y,
                                         float& local) {
   const size_t sl = (size_t)l * o.M * o.N;
-  if (o.trans) {
+  if (!EPI && o.trans) {
     o.C[sl + (size_t)col * o.M + row] = o.ca * y;
     return;
   }
@@ -189,7 +190,7 @@ __device__ __forceinline__ void tile_store(const Out& o, const Fused& f, int i0,
 #pragma unroll
     for (int hj = 0; hj < T::TN / 4; ++hj) {
       const int col = j0 + ftile::tile_col<T>(tx, hj);
-      if (VEC && o.trans) {
+      if (VEC && !EPI && o.trans) {
 #pragma unroll
         for (int l = 0; l < NS; ++l)
 #pragma unroll
@@ -254,7 +255,7 @@ __device__ __forceinline__ void tile_store(const Out& o, const Fused& f, int i0,
           for (int j = 0; j < 4; ++j)
 #pragma unroll
             for (int l = 0; l < NS; ++l)
-              if (col + j < o.N) out_one(o, l, row + i, col + j, y[l][j], loc);
+              if (col + j < o.N) out_one<EPI>(o, l, row + i, col + j, y[l][j], loc);
         }
       }
     }
@@ -341,7 +342,7 @@ __device__ __forceinline__ float split_store(cg::cluster_group& cluster, float* 
 #pragma unroll
           for (int k = 0; k < NS; ++k) y = fmaf(f.epi[l * NS + k], v[k], y);
         }
-        out_one(o, l, row, col, y, local);
+        out_one<EPI>(o, l, row, col, y, local);
       }
     }
   }

@@ -15,9 +15,11 @@
 // that request X_reg: the iterate is then formed from the kept basis at
 // the end (the deferred schedule of lsqr_enqueue), and every kernel here
 // follows that schedule problem by problem.
+#include <algorithm>
 #include <vector>
 
 #include "group.cuh"
+#include "umma.cuh"
 
 namespace {
 
@@ -51,10 +53,14 @@ k_group_norm_c(const GroupProb* __restrict__ probs, double* scal, Layout lay, in
   const int p = blockIdx.y;
   const GroupProb& P = probs[p];
   float s = 0.f;
-  for (size_t i = (size_t)blockIdx.x * GRP_NT + threadIdx.x; i < P.Ty;
-       i += (size_t)gridDim.x * GRP_NT) {
-    const float v = P.C[i];
-    s = fmaf(v, v, s);
+  const size_t st = (size_t)gridDim.x * GRP_NT;
+  for (size_t i0 = (size_t)blockIdx.x * GRP_NT + threadIdx.x; i0 < P.Ty; i0 += 8 * st) {
+    float v[8];  // eight loads in flight a thread
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = i0 + u * st < P.Ty ? __ldg(P.C + i0 + u * st) : 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (i0 + u * st < P.Ty) s = fmaf(v[u], v[u], s);
   }
   Red red;
   red.out = scal + p * lay.stride() + lay.beta();
@@ -221,7 +227,7 @@ bool group_eligible(const std::vector<tc_plan*>& plans, const float* const* C, b
         p->opts.gcv_variant != plans[0]->opts.gcv_variant)
       return false;
     if (prec == TC_BF16 &&
-        (!p->AhL || !p->AhTL || p->n1 % 8 != 0 || p->n2 % 8 != 0 || p->s % 8 != 0))
+        (!p->AhL || !p->AhTL || !p->tmp1 || !p->tmp2 || p->n1 % 8 != 0 || p->n2 % 8 != 0 || p->s % 8 != 0))
       return false;
   }
   if (prec == TC_BF16)  // C is read as float4
@@ -231,7 +237,7 @@ bool group_eligible(const std::vector<tc_plan*>& plans, const float* const* C, b
 }
 
 void group_free(GroupState* g) {
-  void* ps[] = {g->probs, g->scal, g->flags, g->done, g->partials, g->tickets};
+  void* ps[] = {g->probs, g->scal, g->flags, g->done, g->partials, g->tickets, g->maps};
   for (void* q : ps)
     if (q) cudaFree(q);
   for (int c = 0; c < GROUP_CFGS; ++c)
@@ -248,6 +254,7 @@ int group_prepare(GroupState* g, const std::vector<tc_plan*>& plans, const float
   const Layout lay{(size_t)itermax + 2, (size_t)(itermax < TC_MAX_PROJ ? itermax : TC_MAX_PROJ)};
   const int bf16 = plans[0]->opts.precision == TC_BF16, ncfg = group_cfg_count(bf16);
   std::vector<GroupProb> hp(count);
+  std::vector<CUtensorMap> hmaps;
   std::vector<int2> wk[GROUP_CFGS][2];
   size_t npart = 0;
   for (int i = 0; i < count; ++i) {
@@ -255,8 +262,14 @@ int group_prepare(GroupState* g, const std::vector<tc_plan*>& plans, const float
     GroupProb& q = hp[i];
     q.Ah = p->Ah;
     q.AhT = p->AhT;
-    q.AhL = p->AhL;
-    q.AhTL = p->AhTL;
+    if (bf16) {  // the operand buffers of the plan's own products, one each
+      q.opV = p->tmp1;
+      q.opU = p->tmp2;
+      UmmaMaps fm, am;
+      TC_TRY(make_umma_maps(&fm, 0, p->AhL, q.opV, p->n1, p->s, p->n2, p->n3));
+      TC_TRY(make_umma_maps(&am, 0, p->AhTL, q.opU, p->n2, p->s, p->n1, p->n3));
+      hmaps.insert(hmaps.end(), {fm.a, fm.b, am.a, am.b});
+    }
     q.C = C[i];
     q.X = X[i];
     q.Xr = Xr[i];
@@ -274,13 +287,28 @@ int group_prepare(GroupState* g, const std::vector<tc_plan*>& plans, const float
       group_tile_shape(bf16, c, &TM, &TN);
       const int tn = (q.s + TN - 1) / TN;
       const int tf = ((q.n1 + TM - 1) / TM) * tn, ta = ((q.n2 + TM - 1) / TM) * tn;
-      for (int t = 0; t < tf; ++t) wk[c][0].push_back(make_int2(i, t));
-      for (int t = 0; t < ta; ++t) wk[c][1].push_back(make_int2(i, t));
       if ((size_t)tf > most) most = tf;
       if ((size_t)ta > most) most = ta;
     }
     q.partials = reinterpret_cast<double*>(npart);  // offset, made a pointer below
     npart += most;
+  }
+  // Work in the order of falling contraction length: a tile's time follows it, and
+  // the launch's last CTAs are then its shortest (a launch is 5 to 7 waves).
+  for (int d = 0; d < 2; ++d) {
+    auto k_of = [&](int i) { return d == 0 ? hp[i].n2 : hp[i].n1; };
+    std::vector<int> order(count);
+    for (int i = 0; i < count; ++i) order[i] = i;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return k_of(a) > k_of(b); });
+    for (int c = 0; c < ncfg; ++c) {
+      int TM, TN;
+      group_tile_shape(bf16, c, &TM, &TN);
+      for (int i : order) {
+        const int m = d == 0 ? hp[i].n1 : hp[i].n2;
+        const int t = ((m + TM - 1) / TM) * ((hp[i].s + TN - 1) / TN);
+        for (int q = 0; q < t; ++q) wk[c][d].push_back(make_int2(i, q));
+      }
+    }
   }
   TC_TRY(dgrow(&g->probs, &g->probs_n, (size_t)count));
   TC_TRY(dgrow(&g->scal, &g->scal_n, (size_t)count * lay.stride()));
@@ -290,6 +318,11 @@ int group_prepare(GroupState* g, const std::vector<tc_plan*>& plans, const float
   if (!g->tickets || g->tickets_n < (size_t)count) {
     TC_TRY(dgrow(&g->tickets, &g->tickets_n, (size_t)count));
     TC_CUDA(cudaMemsetAsync(g->tickets, 0, (size_t)count * sizeof(unsigned), st));
+  }
+  if (bf16) {
+    TC_TRY(dgrow(&g->maps, &g->maps_n, hmaps.size()));
+    TC_CUDA(cudaMemcpyAsync(g->maps, hmaps.data(), hmaps.size() * sizeof(CUtensorMap),
+                            cudaMemcpyHostToDevice, st));
   }
   for (int c = 0; c < ncfg; ++c)
     for (int d = 0; d < 2; ++d) {
@@ -317,18 +350,6 @@ int group_prepare(GroupState* g, const std::vector<tc_plan*>& plans, const float
 }
 
 namespace {
-int set_tiles(GroupState* g, int cfg) {
-  int TM, TN;
-  group_tile_shape(g->bf16, cfg, &TM, &TN);
-  for (int i = 0; i < g->count; ++i) {
-    GroupProb& q = g->host[i];
-    const int tn = (q.s + TN - 1) / TN;
-    q.tiles_f = ((q.n1 + TM - 1) / TM) * tn;
-    q.tiles_a = ((q.n2 + TM - 1) / TM) * tn;
-  }
-  return TC_OK;
-}
-
 GroupOp make_op(const GroupState* g, int kind, int j) {
   GroupOp o;
   o.op = kind;
@@ -350,8 +371,10 @@ int launch_op(const GroupState* g, const tc_plan* p0, int kind, int j, int cfg, 
   const float* pro = d == 0 ? p0->hM : p0->hMinvT;
   const float* epi = d == 0 ? p0->hMinv : p0->hMT;
   const GroupOp o = make_op(g, kind, j);
-  return g->bf16 ? launch_group_umma(g->probs, g->work[cfg][d], g->nwork[cfg][d], o, pro, epi,
-                                     p0->n3, cfg, st)
+  // BF16: the operand is in place, and the epilogue writes the next product's
+  const float* nxt = d == 0 ? p0->hMinvT : p0->hM;
+  return g->bf16 ? launch_group_umma(g->probs, g->maps, g->work[cfg][d], g->nwork[cfg][d], o, epi,
+                                     nxt, p0->n3, cfg, st)
                  : launch_group_gemm(g->probs, g->work[cfg][d], g->nwork[cfg][d], o, pro, epi,
                                      p0->n3, cfg, st);
 }
@@ -370,9 +393,6 @@ int group_autotune(GroupState* g, const tc_plan* p0, cudaStream_t st) {
   TC_CUDA(cudaEventCreate(&e1));
   for (int c = 0; c < GROUP_CFGS; ++c) g->tune_ms[c] = 0.f;
   for (int c = 0; c < g->ncfg; ++c) {
-    set_tiles(g, c);
-    TC_CUDA(cudaMemcpyAsync(g->probs, g->host.data(), g->host.size() * sizeof(GroupProb),
-                            cudaMemcpyHostToDevice, st));
     TC_TRY(launch_op(g, p0, GOP_FWD, 0, c, st));  // warm-up
     TC_CUDA(cudaEventRecord(e0, st));
     for (int r = 0; r < 3; ++r) TC_TRY(launch_op(g, p0, GOP_FWD, 0, c, st));
@@ -389,22 +409,14 @@ int group_autotune(GroupState* g, const tc_plan* p0, cudaStream_t st) {
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   g->cfg = pick;
-  set_tiles(g, pick);
-  TC_CUDA(cudaMemcpyAsync(g->probs, g->host.data(), g->host.size() * sizeof(GroupProb),
-                          cudaMemcpyHostToDevice, st));
-  TC_CUDA(cudaStreamSynchronize(st));
   return TC_OK;
 }
 
 // Tile shape cfg without timing (tc_batch_info's forced modes).
-int group_fix_tile(GroupState* g, int cfg, cudaStream_t st) {
+int group_fix_tile(GroupState* g, int cfg) {
   TC_CHECK(cfg >= 0 && cfg < g->ncfg);
   for (int c = 0; c < GROUP_CFGS; ++c) g->tune_ms[c] = 0.f;
   g->cfg = cfg;
-  set_tiles(g, cfg);
-  TC_CUDA(cudaMemcpyAsync(g->probs, g->host.data(), g->host.size() * sizeof(GroupProb),
-                          cudaMemcpyHostToDevice, st));
-  TC_CUDA(cudaStreamSynchronize(st));
   return TC_OK;
 }
 
@@ -419,6 +431,12 @@ int group_enqueue(GroupState* g, const tc_plan* p0, double tol, double lambda,
   TC_CUDA(cudaGetLastError());
   k_group_norm_c<<<dim3(NORM_CTAS, count), GRP_NT, 0, st>>>(g->probs, g->scal, lay, g->flags);
   TC_CUDA(cudaGetLastError());
+  if (g->bf16) {
+    size_t most = 0;
+    for (const GroupProb& q : g->host)
+      if ((size_t)q.n1 * q.s > most) most = (size_t)q.n1 * q.s;
+    TC_TRY(launch_group_operand(g->probs, count, most, p0->hMinvT, p0->n3, st));
+  }
   TC_TRY(launch_op(g, p0, GOP_INIT, 0, c, st));
   k_group_lsqr_init<<<tb, 128, 0, st>>>(g->scal, lay, g->flags, g->done, count);
   TC_CUDA(cudaGetLastError());

@@ -70,6 +70,8 @@ struct GroupState {
   int* done = nullptr;
   double* partials = nullptr;
   unsigned* tickets = nullptr;
+  struct CUtensorMap_st* maps = nullptr;  // BF16: four a problem
+  size_t maps_n = 0;
   int bf16 = 0;                      // 1: BF16 plans (group_tc.cu), 0: FP32 (gemm.cu)
   int ncfg = 0;                      // tile shapes the autotuner times
   int2* work[GROUP_CFGS][2] = {};    // [tile shape][forward, adjoint]
@@ -88,7 +90,7 @@ bool group_eligible(const std::vector<tc_plan*>& plans, const float* const* C, b
 int group_prepare(GroupState* g, const std::vector<tc_plan*>& plans, const float* const* C,
                   float* const* X, float* const* Xr, int itermax, cudaStream_t st);
 int group_autotune(GroupState* g, const tc_plan* p0, cudaStream_t st);
-int group_fix_tile(GroupState* g, int cfg, cudaStream_t st);
+int group_fix_tile(GroupState* g, int cfg);
 int group_enqueue(GroupState* g, const tc_plan* p0, double tol, double lambda,
                   tc_solve_info* infos, cudaStream_t st);
 void group_free(GroupState* g);

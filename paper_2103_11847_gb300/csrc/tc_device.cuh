@@ -41,8 +41,9 @@ __device__ __forceinline__ double rsqrt_newton(double x) {
 // (ca, cp) of the epilogue rule, computed by thread 0 in FP64 and broadcast.
 // A zero denominator gives a zero coefficient: that is how a Golub-Kahan
 // breakdown (beta or alpha = 0) produces a zero tensor instead of Inf/NaN.
-__device__ __forceinline__ void coef_compute(const Coef& c, float* sh2) {
-  if (threadIdx.x == 0 && threadIdx.y == 0) {
+// coef_compute_by: by thread `who`.
+__device__ __forceinline__ void coef_compute_by(const Coef& c, float* sh2, unsigned who) {
+  if (threadIdx.x == who && threadIdx.y == 0) {
     double ca = 1.0, cp = 0.0;
     switch (c.rule) {
       case COEF_RESID: ca = -1.0; cp = 1.0; break;
@@ -66,6 +67,7 @@ __device__ __forceinline__ void coef_compute(const Coef& c, float* sh2) {
     sh2[1] = (float)cp;
   }
 }
+__device__ __forceinline__ void coef_compute(const Coef& c, float* sh2) { coef_compute_by(c, sh2, 0); }
 
 // Programmatic dependent launch. A kernel launched with the programmatic
 // stream-serialization attribute may start while its predecessor finishes;

@@ -359,8 +359,8 @@ int tc_kernels_init();
 struct GroupProb {
   const float* Ah = nullptr;   // A~ (n1 x n2 a slice) and its slice transposes
   const float* AhT = nullptr;
-  const void* AhL = nullptr;   // BF16 plans: the same rounded to BF16
-  const void* AhTL = nullptr;
+  void* opV = nullptr;         // BF16 plans: the forward product's operand, bf16(V~ x_3 M)
+  void* opU = nullptr;         // and the adjoint's, bf16(U~ x_3 M^{-T}), from the product before
   const float* C = nullptr;
   float* X = nullptr;
   float* Xr = nullptr;
@@ -371,7 +371,6 @@ struct GroupProb {
   unsigned* ticket = nullptr;  // and arrival ticket
   size_t Tx = 0, Ty = 0;
   int n1 = 0, n2 = 0, s = 0;
-  int tiles_f = 0, tiles_a = 0;  // CTAs of the forward (M = n1) / adjoint (M = n2) product
   int pad = 0;
 };
 // The state of one grouped launch: which product, the step, and the
@@ -392,15 +391,21 @@ struct GroupOp {
 // (problem, tile) for CTA i. Tile shape cfg (0 .. group_cfg_count - 1) is
 // group_tile_shape's tm x tn output tile:
 // * gemm.cu, FP32 plans: FFMA, three shapes;
-// * group_tc.cu, BF16 plans: tcgen05 with the transforms in the operand load
-//   and the epilogue, two shapes.
+// * group_tc.cu, BF16 plans: tcgen05, the epilogue with the trailing transform
+//   and the next product's operand, two shapes. maps: four tensor maps a problem
+//   (A~ and opV for the forward product, A~^T and opU for the adjoint).
 #define GROUP_CFGS 3
 int group_cfg_count(int bf16);
 void group_tile_shape(int bf16, int cfg, int* tm, int* tn);
 int launch_group_gemm(const GroupProb* probs, const int2* work, int nwork, const GroupOp& g,
                       const float* pro, const float* epi, int n3, int cfg, cudaStream_t st);
-int launch_group_umma(const GroupProb* probs, const int2* work, int nwork, const GroupOp& g,
-                      const float* pro, const float* epi, int n3, int cfg, cudaStream_t st);
+int launch_group_umma(const GroupProb* probs, const struct CUtensorMap_st* maps, const int2* work,
+                      int nwork, const GroupOp& g, const float* epi, const float* nxt, int n3,
+                      int cfg, cudaStream_t st);
+// opU = bf16(C x_3 T) of every problem, the first adjoint product's operand
+// (nxt: T; most: the largest problem's pixels).
+int launch_group_operand(const GroupProb* probs, int count, size_t most, const float* nxt, int n3,
+                         cudaStream_t st);
 int group_tc_init();
 
 // solvers.cu: the c-LSQR solve as a sequence of launches on one stream
