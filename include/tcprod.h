@@ -242,7 +242,8 @@ int tc_gmres_c(tc_plan* plan, const float* C, const float* X0, float* X,
  *    tile) work table, each problem's own scalars, flags and deterministic
  *    reductions), about 3 itermax + 10 launches a batch. The products fuse
  *    both mode-3 transforms: FFMA tiles for FP32 plans, tcgen05 tiles (BF16
- *    operands, FP32 accumulation) for BF16 plans. The tile shape is chosen
+ *    operands, FP32 accumulation; the leading transform in the epilogue of
+ *    the product before) for BF16 plans. The tile shape is chosen
  *    on the first call by timing each candidate on the batch's forward
  *    product. Results equal tc_lsqr_c's up to the order of FP32 additions
  *    (the single solve may split K over a cluster, or run the BF16 transform

@@ -11,7 +11,8 @@
 // and the whole grouped solve is captured once as a CUDA graph.
 //
 // It serves batches of FP32 or BF16 plans with n3 <= 4 (the products fuse
-// the mode-3 transforms: gemm.cu's FFMA tiles, group_tc.cu's tcgen05 tiles)
+// the mode-3 transforms: gemm.cu's FFMA tiles; group_tc.cu's tcgen05 tiles, whose
+// epilogue also writes the next product's BF16 operand)
 // that request X_reg: the iterate is then formed from the kept basis at
 // the end (the deferred schedule of lsqr_enqueue), and every kernel here
 // follows that schedule problem by problem.
