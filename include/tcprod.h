@@ -263,9 +263,9 @@ int tc_lsqr_c_batched(tc_batch* batch, const float* const* C, float* const* X,
  * solve); -1: unchanged. Writes (host, each may be NULL) whether the last
  * solve ran grouped, the tile shape in use (-1 before the first grouped
  * solve) and the candidates' forward-product times in ms (tune_ms[3], zero
- * where not timed). Tile shapes: FP32 plans 0: 64 x 64 in K blocks of 16, 1:
- * 64 x 64 in K blocks of 8, 2: 128 x 64 (results the same to the bit); BF16
- * plans 0: 128 x 64, 1: 128 x 128. */
+ * where not timed). Tile shapes: FP32 plans 0: 64 x 64, 1: 32 x 32, 2: 128 x 64
+ * (0 and 2 the same to the bit); BF16 plans 0: 128 x 64, 1: 128 x 128 (the same
+ * to the bit). */
 int tc_batch_info(tc_batch* batch, int mode, int* grouped, int* tile, float* tune_ms);
 
 /* ---- Learned lambda and stopping index --------------------------------------

@@ -496,11 +496,52 @@ k_group_gemm(const GroupProb* __restrict__ probs, const int2* __restrict__ work,
                       (unsigned)((M + 63) / 64 * tn));
 }
 
-// Tile shapes the autotuner chooses from: cfg 0: 64 x 64 (128 threads, K
-// blocks of 16), 1: 64 x 64 (K blocks of 8: less shared memory), 2: 128 x 64
-// (256 threads). All give the same bits.
+// The same with 32 x 32 tiles (small_tile_mainloop), stored from the registers:
+// batches whose 64 x 64 tiles are too few for the SMs (30 problems of n in
+// 64..128: 347 us a solve of 6 steps against 360 with 64 x 64 tiles).
+template <int NS>
+__global__ void __launch_bounds__(128)
+k_group_small(const GroupProb* __restrict__ probs, const int2* __restrict__ work, GroupOp g,
+              Fused f) {
+  constexpr int BM = 32, BN = 32, BK = 16, TM = 4, TN = 2;
+  const int2 w = work[blockIdx.x];
+  const GroupProb& P = probs[w.x];
+  if (g.op != GOP_INIT && g.done[(size_t)w.x * g.lstride + g.j]) return;  // uniform over the problem's CTAs
+  __shared__ __align__(16) float sm[SmallSmem<NS, BM, BN, BK>::kMain];
+  __shared__ float sh_coef[2];
+  const GroupOperands o = group_operands(P, g, w.x);
+  const int M = o.M, K = o.K, N = o.N;
+  const int tn = (N + BN - 1) / BN;
+  const int i0 = (w.y / tn) * BM, j0 = (w.y % tn) * BN;
+  float acc[NS][TM][TN];
+  small_tile_mainloop<NS, BM, BN, BK, TM, TN, true>(o.fwd ? P.AhT : P.Ah, o.B, M, N, K, 0, K, i0, j0,
+                                                    f, sm, acc);
+  coef_compute(o.coef, sh_coef);
+  __syncthreads();
+  const Out out{o.C, o.prev, nullptr, true, false, M, N, sh_coef[0], sh_coef[1]};
+  const int tx = threadIdx.x % (BN / TN), ty = threadIdx.x / (BN / TN);
+  float local = 0.f;
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) {
+      const int row = i0 + ty * TM + i, col = j0 + tx * TN + j;
+      if (row >= M || col >= N) continue;
+#pragma unroll
+      for (int l = 0; l < NS; ++l) {
+        float y = 0.f;
+#pragma unroll
+        for (int k = 0; k < NS; ++k) y = fmaf(f.epi[l * NS + k], acc[k][i][j], y);
+        out_one<true>(out, l, row, col, y, local);
+      }
+    }
+  reduce_finish_n(local, o.red, (unsigned)w.y, (unsigned)((M + BM - 1) / BM * tn));
+}
+
+// Tile shapes the autotuner chooses from: cfg 0: 64 x 64 (128 threads), 1: 32 x 32
+// (k_group_small), 2: 128 x 64 (256 threads). 0 and 2 give the same bits.
 template <int NS, int CFG>
-using GroupTile = ftile::Tile<NS, CFG == 2 ? 128 : 64, 64, CFG == 1 ? 8 : 16, 4, 3, true>;
+using GroupTile = ftile::Tile<NS, CFG == 2 ? 128 : 64, 64, 16, 4, 3, true>;
 
 template <class K>
 int allow_smem(K kernel, size_t bytes) {
@@ -513,8 +554,12 @@ int allow_smem(K kernel, size_t bytes) {
 template <int NS, int CFG>
 int run_group(const GroupProb* probs, const int2* work, int nwork, const GroupOp& g,
               const Fused& f, cudaStream_t st) {
-  using T = GroupTile<NS, CFG>;
-  k_group_gemm<T><<<nwork, T::NT, T::bytes, st>>>(probs, work, g, f);
+  if constexpr (CFG == 1) {
+    k_group_small<NS><<<nwork, 128, 0, st>>>(probs, work, g, f);
+  } else {
+    using T = GroupTile<NS, CFG>;
+    k_group_gemm<T><<<nwork, T::NT, T::bytes, st>>>(probs, work, g, f);
+  }
   TC_CUDA(cudaGetLastError());
   return TC_OK;
 }
@@ -649,7 +694,6 @@ int init_ns() {
   TC_TRY((init_fused<TileM<NS>, true, false, true>()));
   TC_TRY((init_fused<TileM<NS>, false, true, true>()));
   TC_TRY(allow_smem(k_group_gemm<GroupTile<NS, 0>>, GroupTile<NS, 0>::bytes));
-  TC_TRY(allow_smem(k_group_gemm<GroupTile<NS, 1>>, GroupTile<NS, 1>::bytes));
   return allow_smem(k_group_gemm<GroupTile<NS, 2>>, GroupTile<NS, 2>::bytes);
 }
 
@@ -662,8 +706,8 @@ void group_tile_shape(int bf16, int cfg, int* tm, int* tn) {
     *tm = 128;
     *tn = cfg == 1 ? 128 : 64;
   } else {
-    *tm = cfg == 2 ? 128 : 64;
-    *tn = 64;
+    *tm = cfg == 2 ? 128 : (cfg == 1 ? 32 : 64);
+    *tn = cfg == 1 ? 32 : 64;
   }
 }
 
