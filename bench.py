@@ -411,7 +411,8 @@ def dual_route_form(A, C, Xt, s, iters, dev, peaks, steps):
                                   du_bytes)}
 
 
-GROUP_TILES = {0: ["64x64 FFMA tiles of 4x4", "32x32 FFMA tiles of 4x2", "64x64 FFMA tiles of 8x4"],
+GROUP_TILES = {0: ["64x64 packed-FMA tiles of 8x4", "32x32 FFMA tiles of 4x2",
+                   "128x64 packed-FMA tiles of 8x4"],
                1: ["128x64 tcgen05 tiles", "128x128 tcgen05 tiles"]}
 
 
