@@ -49,10 +49,15 @@ struct SmallSmem {
 // The main loop of one small fused tile: acc[k] += A_k (pro B)_k over K range
 // [kbeg, kend) for the BM x BN tile at (i0, j0), all NS slices, with register
 // double buffering (the next K tile's global loads are issued before the
-// current tile's FMAs). At is K-major (K x M a slice). One float4 per thread
-// and slice for each of the A and B tiles (vec: 16-byte aligned rows of whole
-// groups). sm: the SmallSmem floats.
-template <int NS, int BM, int BN, int BK, int TM, int TN, bool PRO>
+// current tile's FMAs). At is K-major (K x M a slice). Four values of each of the
+// A and B tiles a thread and slice. VEC: both operands have 16-byte aligned rows
+// of whole groups of four; otherwise each operand is looked at by itself, and one
+// that has not is read value by value, a warp's lanes side by side. The choice is
+// a template parameter, or one branch around all of an operand's loads: a branch
+// around each load kept the compiler from issuing them together (n3 = 4, c-LSQR
+// of 2048 x 2048 with 64 columns: 1702 us a solve of 6 steps, now 1480; of 1600 x
+// 200 with 24 columns: 344, now 298). sm: the SmallSmem floats.
+template <int NS, int BM, int BN, int BK, int TM, int TN, bool PRO, bool VEC>
 __device__ __forceinline__ void small_tile_mainloop(const float* __restrict__ At,
                                                     const float* __restrict__ B, int M, int N,
                                                     int K, int kbeg, int kend, int i0, int j0,
@@ -72,37 +77,48 @@ __device__ __forceinline__ void small_tile_mainloop(const float* __restrict__ At
 #pragma unroll
       for (int j = 0; j < TN; ++j) acc[k][i][j] = 0.f;
 
-  static_assert(BM * BK == 4 * NT && BK * BN == 4 * NT, "one float4 per thread per tile");
-  const bool vec = ((M | N) % 4 == 0) && ((reinterpret_cast<uintptr_t>(At) |
-                                           reinterpret_cast<uintptr_t>(B)) & 15) == 0;
-  const int ar = tid / (BM / 4), ac = (tid % (BM / 4)) * 4;  // A tile: K row, first output row
-  const int br = tid / (BN / 4), bc = (tid % (BN / 4)) * 4;  // B tile: K row, first column
+  static_assert(BM * BK == 4 * NT && BK * BN == 4 * NT, "four values a thread of each tile");
+  auto whole = [](const float* p, int cols) {
+    return cols % 4 == 0 && (reinterpret_cast<uintptr_t>(p) & 15) == 0;
+  };
+  const bool va = VEC || whole(At, M), vb = VEC || whole(B, N);
+  // A thread's four values are positions 4 tid .. + 3 of the tile (vec), else
+  // tid, tid + NT, ..; position p is K row p / W, column p % W
   float4 ra[NS], rb[NS];
-  auto load4 = [&](const float* src, int c, int cols) {
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (vec && c + 3 < cols) {
-      v = __ldg(reinterpret_cast<const float4*>(src + c));
+  auto load = [&](float4 (&r)[NS], const float* base, size_t slice, int cols, int k0, int c0,
+                  int W, bool vec) {
+    if (vec) {
+      const int row = k0 + 4 * tid / W, c = c0 + 4 * tid % W;
+      const bool in = row < kend && c < cols;
+      const float* src = base + (size_t)row * cols + c;
+#pragma unroll
+      for (int k = 0; k < NS; ++k)
+        r[k] = in ? __ldg(reinterpret_cast<const float4*>(src + k * slice))
+                  : make_float4(0.f, 0.f, 0.f, 0.f);
     } else {
-      v.x = c < cols ? __ldg(src + c) : 0.f;
-      v.y = c + 1 < cols ? __ldg(src + c + 1) : 0.f;
-      v.z = c + 2 < cols ? __ldg(src + c + 2) : 0.f;
-      v.w = c + 3 < cols ? __ldg(src + c + 3) : 0.f;
+      auto one = [&](int k, int e) {
+        const int row = k0 + (tid + NT * e) / W, c = c0 + (tid + NT * e) % W;
+        return row < kend && c < cols ? __ldg(base + k * slice + (size_t)row * cols + c) : 0.f;
+      };
+#pragma unroll
+      for (int k = 0; k < NS; ++k) r[k] = make_float4(one(k, 0), one(k, 1), one(k, 2), one(k, 3));
     }
-    return v;
+  };
+  auto store = [&](float* tile, const float4& v, bool vec) {
+    if (vec) {
+      *reinterpret_cast<float4*>(tile + 4 * tid) = v;
+    } else {
+      tile[tid] = v.x; tile[tid + NT] = v.y; tile[tid + 2 * NT] = v.z; tile[tid + 3 * NT] = v.w;
+    }
   };
   auto fetch = [&](int k0) {
-#pragma unroll
-    for (int k = 0; k < NS; ++k) {
-      ra[k] = k0 + ar < kend ? load4(At + k * sA + (size_t)(k0 + ar) * M, i0 + ac, M)
-                             : make_float4(0.f, 0.f, 0.f, 0.f);
-      rb[k] = k0 + br < kend ? load4(B + k * sB + (size_t)(k0 + br) * N, j0 + bc, N)
-                             : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    load(ra, At, sA, M, k0, i0, BM, va);
+    load(rb, B, sB, N, k0, j0, BN, vb);
   };
   if (kbeg < kend) fetch(kbeg);
   for (int k0 = kbeg; k0 < kend; k0 += BK) {
 #pragma unroll
-    for (int k = 0; k < NS; ++k) *reinterpret_cast<float4*>(&As[k][ar][ac]) = ra[k];
+    for (int k = 0; k < NS; ++k) store(&As[k][0][0], ra[k], va);
     if (PRO) {
 #pragma unroll
       for (int k = 0; k < NS; ++k) {
@@ -115,11 +131,11 @@ __device__ __forceinline__ void small_tile_mainloop(const float* __restrict__ At
           t.z = fmaf(m, rb[l].z, t.z);
           t.w = fmaf(m, rb[l].w, t.w);
         }
-        *reinterpret_cast<float4*>(&Bs[k][br][bc]) = t;
+        store(&Bs[k][0][0], t, vb);
       }
     } else {
 #pragma unroll
-      for (int l = 0; l < NS; ++l) *reinterpret_cast<float4*>(&Bs[l][br][bc]) = rb[l];
+      for (int l = 0; l < NS; ++l) store(&Bs[l][0][0], rb[l], vb);
     }
     __syncthreads();
     if (k0 + BK < kend) fetch(k0 + BK);
@@ -351,7 +367,7 @@ __device__ __forceinline__ float split_store(cg::cluster_group& cluster, float* 
 
 // Small fused tiles, K split over the cluster (a cluster of one: no split);
 // the epilogue runs from the summed partial tiles.
-template <int NS, int BM, int BN, int BK, int TM, int TN, bool PRO, bool EPI>
+template <int NS, int BM, int BN, int BK, int TM, int TN, bool PRO, bool EPI, bool VEC>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN))
 k_fused_small(const float* __restrict__ At, const float* __restrict__ B, float* C, int M, int N,
               int K, int kchunk, Fused f, Epi ep, int trans) {
@@ -370,7 +386,8 @@ k_fused_small(const float* __restrict__ At, const float* __restrict__ B, float* 
   const int kend = min(K, kbeg + kchunk);
 
   float acc[NS][TM][TN];
-  small_tile_mainloop<NS, BM, BN, BK, TM, TN, PRO>(At, B, M, N, K, kbeg, kend, i0, j0, f, sm, acc);
+  small_tile_mainloop<NS, BM, BN, BK, TM, TN, PRO, VEC>(At, B, M, N, K, kbeg, kend, i0, j0, f, sm,
+                                                       acc);
   // partial tile to shared memory, then sum over the cluster's K ranges
 #pragma unroll
   for (int k = 0; k < NS; ++k)
@@ -514,8 +531,13 @@ k_group_small(const GroupProb* __restrict__ probs, const int2* __restrict__ work
   const int tn = (N + BN - 1) / BN;
   const int i0 = (w.y / tn) * BM, j0 = (w.y % tn) * BN;
   float acc[NS][TM][TN];
-  small_tile_mainloop<NS, BM, BN, BK, TM, TN, true>(o.fwd ? P.AhT : P.Ah, o.B, M, N, K, 0, K, i0, j0,
-                                                    f, sm, acc);
+  const float* At = o.fwd ? P.AhT : P.Ah;
+  const bool vec = (M | N) % 4 == 0 &&  // uniform over the problem's CTAs
+                   ((reinterpret_cast<uintptr_t>(At) | reinterpret_cast<uintptr_t>(o.B)) & 15) == 0;
+  if (vec)
+    small_tile_mainloop<NS, BM, BN, BK, TM, TN, true, true>(At, o.B, M, N, K, 0, K, i0, j0, f, sm, acc);
+  else
+    small_tile_mainloop<NS, BM, BN, BK, TM, TN, true, false>(At, o.B, M, N, K, 0, K, i0, j0, f, sm, acc);
   coef_compute(o.coef, sh_coef);
   __syncthreads();
   const Out out{o.C, o.prev, nullptr, true, false, M, N, sh_coef[0], sh_coef[1]};
@@ -645,8 +667,11 @@ int pick_tile(const float* At, const float* B, float* C, int M, int N, int K, co
   const long tiles = (long)((M + 31) / 32) * ((N + 31) / 32);
   while (KS < 8 && tiles * KS < NSM && K >= 2 * BK * (KS * 2)) KS *= 2;
   const int kchunk = (((K + KS - 1) / KS) + BK - 1) / BK * BK;
-  return launch_cluster(k_fused_small<NS, 32, 32, BK, 4, 2, PRO, EPI>, 32, 32, 128, 0, KS, At, B, C,
-                        M, N, K, kchunk, f, ep, trans, st);
+  const bool vec = (M | N) % 4 == 0 && al16(At) && al16(B);
+  return vec ? launch_cluster(k_fused_small<NS, 32, 32, BK, 4, 2, PRO, EPI, true>, 32, 32, 128, 0, KS,
+                              At, B, C, M, N, K, kchunk, f, ep, trans, st)
+             : launch_cluster(k_fused_small<NS, 32, 32, BK, 4, 2, PRO, EPI, false>, 32, 32, 128, 0, KS,
+                              At, B, C, M, N, K, kchunk, f, ep, trans, st);
 }
 
 template <int NS>
