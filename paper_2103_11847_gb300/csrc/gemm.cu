@@ -46,17 +46,33 @@ struct SmallSmem {
   static constexpr int kFloats = kMain > kPart ? kMain : kPart;
 };
 
+// Predicated loads, zero where !ok: no branch, so that a thread's loads issue together.
+__device__ __forceinline__ float4 ldg4_if(const float* p, bool ok) {
+  float4 v;
+  asm("{\n .reg .pred q;\n setp.ne.u32 q, %5, 0;\n mov.b32 %0, 0;\n mov.b32 %1, 0;\n"
+      " mov.b32 %2, 0;\n mov.b32 %3, 0;\n @q ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];\n}"
+      : "=&f"(v.x), "=&f"(v.y), "=&f"(v.z), "=&f"(v.w)
+      : "l"(p), "r"((unsigned)ok));
+  return v;
+}
+__device__ __forceinline__ float ldg_if(const float* p, bool ok) {
+  float v;
+  asm("{\n .reg .pred q;\n setp.ne.u32 q, %2, 0;\n mov.b32 %0, 0;\n @q ld.global.nc.f32 %0, [%1];\n}"
+      : "=&f"(v)
+      : "l"(p), "r"((unsigned)ok));
+  return v;
+}
+
 // The main loop of one small fused tile: acc[k] += A_k (pro B)_k over K range
 // [kbeg, kend) for the BM x BN tile at (i0, j0), all NS slices, with register
 // double buffering (the next K tile's global loads are issued before the
 // current tile's FMAs). At is K-major (K x M a slice). Four values of each of the
 // A and B tiles a thread and slice. VEC: both operands have 16-byte aligned rows
 // of whole groups of four; otherwise each operand is looked at by itself, and one
-// that has not is read value by value, a warp's lanes side by side. The choice is
-// a template parameter, or one branch around all of an operand's loads: a branch
-// around each load kept the compiler from issuing them together (n3 = 4, c-LSQR
-// of 2048 x 2048 with 64 columns: 1702 us a solve of 6 steps, now 1480; of 1600 x
-// 200 with 24 columns: 344, now 298). sm: the SmallSmem floats.
+// that has not is read value by value, a warp's lanes side by side. The loads are
+// predicated: as branches they kept the compiler from issuing them together
+// (c-LSQR of 6 steps at n3 = 4: 1600 x 200 with 24 columns 344 us, now 298; 2048
+// x 2048 with 64 columns 1702, now 1446). sm: the SmallSmem floats.
 template <int NS, int BM, int BN, int BK, int TM, int TN, bool PRO, bool VEC>
 __device__ __forceinline__ void small_tile_mainloop(const float* __restrict__ At,
                                                     const float* __restrict__ B, int M, int N,
@@ -82,43 +98,44 @@ __device__ __forceinline__ void small_tile_mainloop(const float* __restrict__ At
     return cols % 4 == 0 && (reinterpret_cast<uintptr_t>(p) & 15) == 0;
   };
   const bool va = VEC || whole(At, M), vb = VEC || whole(B, N);
-  // A thread's four values are positions 4 tid .. + 3 of the tile (vec), else
-  // tid, tid + NT, ..; position p is K row p / W, column p % W
+  const int ar = tid / (BM / 4), ac = (tid % (BM / 4)) * 4;  // A tile: K row, first output row
+  const int br = tid / (BN / 4), bc = (tid % (BN / 4)) * 4;  // B tile: K row, first column
+  // A thread's four values: those at (row, col) of the tile and after it (vec),
+  // else positions tid, tid + NT, .. of the tile
   float4 ra[NS], rb[NS];
-  auto load = [&](float4 (&r)[NS], const float* base, size_t slice, int cols, int k0, int c0,
-                  int W, bool vec) {
+  auto load = [&](float4 (&r)[NS], const float* base, size_t slice, int cols, int k0, int c0, int W,
+                  int row, int col, bool vec) {
     if (vec) {
-      const int row = k0 + 4 * tid / W, c = c0 + 4 * tid % W;
-      const bool in = row < kend && c < cols;
-      const float* src = base + (size_t)row * cols + c;
+      const int kr = k0 + row, c = c0 + col;
+      const bool in = kr < kend && c < cols;
+      const float* src = base + (size_t)kr * cols + c;
 #pragma unroll
-      for (int k = 0; k < NS; ++k)
-        r[k] = in ? __ldg(reinterpret_cast<const float4*>(src + k * slice))
-                  : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int k = 0; k < NS; ++k) r[k] = ldg4_if(src + k * slice, in);
     } else {
       auto one = [&](int k, int e) {
-        const int row = k0 + (tid + NT * e) / W, c = c0 + (tid + NT * e) % W;
-        return row < kend && c < cols ? __ldg(base + k * slice + (size_t)row * cols + c) : 0.f;
+        const int kr = k0 + (tid + NT * e) / W, c = c0 + (tid + NT * e) % W;
+        return ldg_if(base + k * slice + (size_t)kr * cols + c, kr < kend && c < cols);
       };
 #pragma unroll
       for (int k = 0; k < NS; ++k) r[k] = make_float4(one(k, 0), one(k, 1), one(k, 2), one(k, 3));
     }
   };
-  auto store = [&](float* tile, const float4& v, bool vec) {
+  // at: the thread's (row, col); tile: the slice's first value
+  auto store = [&](float* at, float* tile, const float4& v, bool vec) {
     if (vec) {
-      *reinterpret_cast<float4*>(tile + 4 * tid) = v;
+      *reinterpret_cast<float4*>(at) = v;
     } else {
       tile[tid] = v.x; tile[tid + NT] = v.y; tile[tid + 2 * NT] = v.z; tile[tid + 3 * NT] = v.w;
     }
   };
   auto fetch = [&](int k0) {
-    load(ra, At, sA, M, k0, i0, BM, va);
-    load(rb, B, sB, N, k0, j0, BN, vb);
+    load(ra, At, sA, M, k0, i0, BM, ar, ac, va);
+    load(rb, B, sB, N, k0, j0, BN, br, bc, vb);
   };
   if (kbeg < kend) fetch(kbeg);
   for (int k0 = kbeg; k0 < kend; k0 += BK) {
 #pragma unroll
-    for (int k = 0; k < NS; ++k) store(&As[k][0][0], ra[k], va);
+    for (int k = 0; k < NS; ++k) store(&As[k][ar][ac], &As[k][0][0], ra[k], va);
     if (PRO) {
 #pragma unroll
       for (int k = 0; k < NS; ++k) {
@@ -131,11 +148,11 @@ __device__ __forceinline__ void small_tile_mainloop(const float* __restrict__ At
           t.z = fmaf(m, rb[l].z, t.z);
           t.w = fmaf(m, rb[l].w, t.w);
         }
-        store(&Bs[k][0][0], t, vb);
+        store(&Bs[k][br][bc], &Bs[k][0][0], t, vb);
       }
     } else {
 #pragma unroll
-      for (int l = 0; l < NS; ++l) store(&Bs[l][0][0], rb[l], vb);
+      for (int l = 0; l < NS; ++l) store(&Bs[l][br][bc], &Bs[l][0][0], rb[l], vb);
     }
     __syncthreads();
     if (k0 + BK < kend) fetch(k0 + BK);
@@ -366,9 +383,14 @@ __device__ __forceinline__ float split_store(cg::cluster_group& cluster, float* 
 }
 
 // Small fused tiles, K split over the cluster (a cluster of one: no split);
-// the epilogue runs from the summed partial tiles.
+// the epilogue runs from the summed partial tiles. Read value by value (!VEC) four
+// CTAs a SM are asked for: left to itself the compiler there saves the registers
+// that the next K block's loads need (M x K x N x n3 130 x 800 x 200 x 1 8.5 us
+// with it not asked for, 8.2 with; 512 x 800 x 330 x 3 69.5 and 61.7). With whole
+// groups it costs long narrow products more than it gives others (c-LSQR of 2048 x
+// 2048 with 64 columns, n3 = 4: 1446 us, asked for 1813).
 template <int NS, int BM, int BN, int BK, int TM, int TN, bool PRO, bool EPI, bool VEC>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN))
+__global__ void __launch_bounds__((BM / TM) * (BN / TN), VEC ? 0 : 4)
 k_fused_small(const float* __restrict__ At, const float* __restrict__ B, float* C, int M, int N,
               int K, int kchunk, Fused f, Epi ep, int trans) {
   constexpr int TX = BN / TN;
