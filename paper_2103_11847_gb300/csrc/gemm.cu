@@ -63,17 +63,23 @@ __device__ __forceinline__ float ldg_if(const float* p, bool ok) {
   return v;
 }
 
+// How the small tiles read their operands: LD_BRANCH, a branch a load on whole
+// groups in both operands; LD_WHOLE, predicated, whole groups in both; LD_EACH,
+// predicated, each operand by its own alignment.
+enum Loads { LD_BRANCH, LD_WHOLE, LD_EACH };
+
 // The main loop of one small fused tile: acc[k] += A_k (pro B)_k over K range
 // [kbeg, kend) for the BM x BN tile at (i0, j0), all NS slices, with register
 // double buffering (the next K tile's global loads are issued before the
 // current tile's FMAs). At is K-major (K x M a slice). Four values of each of the
-// A and B tiles a thread and slice. VEC: both operands have 16-byte aligned rows
-// of whole groups of four; otherwise each operand is looked at by itself, and one
-// that has not is read value by value, a warp's lanes side by side. The loads are
-// predicated: as branches they kept the compiler from issuing them together
-// (c-LSQR of 6 steps at n3 = 4: 1600 x 200 with 24 columns 344 us, now 298; 2048
-// x 2048 with 64 columns 1702, now 1446). sm: the SmallSmem floats.
-template <int NS, int BM, int BN, int BK, int TM, int TN, bool PRO, bool VEC>
+// A and B tiles a thread and slice. Single products take the predicated loads:
+// 16-byte ones where an operand has aligned rows of whole groups of four, else value
+// by value, a warp's lanes side by side. Branches kept the compiler from issuing
+// them together (c-LSQR of 6 steps at n3 = 4: 1600 x 200 with 24 columns 344 us,
+// now 298; 2048 x 2048 with 64 columns 1702, now 1446). The grouped form keeps the
+// branches: its tile shape is chosen by time, and a batch's last bits follow the
+// shape. sm: the SmallSmem floats.
+template <int NS, int BM, int BN, int BK, int TM, int TN, bool PRO, Loads LD>
 __device__ __forceinline__ void small_tile_mainloop(const float* __restrict__ At,
                                                     const float* __restrict__ B, int M, int N,
                                                     int K, int kbeg, int kend, int i0, int j0,
@@ -97,7 +103,9 @@ __device__ __forceinline__ void small_tile_mainloop(const float* __restrict__ At
   auto whole = [](const float* p, int cols) {
     return cols % 4 == 0 && (reinterpret_cast<uintptr_t>(p) & 15) == 0;
   };
-  const bool va = VEC || whole(At, M), vb = VEC || whole(B, N);
+  const bool both = (M | N) % 4 == 0 && ((reinterpret_cast<uintptr_t>(At) |
+                                          reinterpret_cast<uintptr_t>(B)) & 15) == 0;
+  const bool va = LD == LD_EACH ? whole(At, M) : true, vb = LD == LD_EACH ? whole(B, N) : true;
   const int ar = tid / (BM / 4), ac = (tid % (BM / 4)) * 4;  // A tile: K row, first output row
   const int br = tid / (BN / 4), bc = (tid % (BN / 4)) * 4;  // B tile: K row, first column
   // A thread's four values: those at (row, col) of the tile and after it (vec),
@@ -128,9 +136,31 @@ __device__ __forceinline__ void small_tile_mainloop(const float* __restrict__ At
       tile[tid] = v.x; tile[tid + NT] = v.y; tile[tid + 2 * NT] = v.z; tile[tid + 3 * NT] = v.w;
     }
   };
+  auto load4 = [&](const float* src, int c, int cols) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (both && c + 3 < cols) {
+      v = __ldg(reinterpret_cast<const float4*>(src + c));
+    } else {
+      v.x = c < cols ? __ldg(src + c) : 0.f;
+      v.y = c + 1 < cols ? __ldg(src + c + 1) : 0.f;
+      v.z = c + 2 < cols ? __ldg(src + c + 2) : 0.f;
+      v.w = c + 3 < cols ? __ldg(src + c + 3) : 0.f;
+    }
+    return v;
+  };
   auto fetch = [&](int k0) {
-    load(ra, At, sA, M, k0, i0, BM, ar, ac, va);
-    load(rb, B, sB, N, k0, j0, BN, br, bc, vb);
+    if constexpr (LD == LD_BRANCH) {
+#pragma unroll
+      for (int k = 0; k < NS; ++k) {
+        ra[k] = k0 + ar < kend ? load4(At + k * sA + (size_t)(k0 + ar) * M, i0 + ac, M)
+                               : make_float4(0.f, 0.f, 0.f, 0.f);
+        rb[k] = k0 + br < kend ? load4(B + k * sB + (size_t)(k0 + br) * N, j0 + bc, N)
+                               : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    } else {
+      load(ra, At, sA, M, k0, i0, BM, ar, ac, va);
+      load(rb, B, sB, N, k0, j0, BN, br, bc, vb);
+    }
   };
   if (kbeg < kend) fetch(kbeg);
   for (int k0 = kbeg; k0 < kend; k0 += BK) {
@@ -408,8 +438,8 @@ k_fused_small(const float* __restrict__ At, const float* __restrict__ B, float* 
   const int kend = min(K, kbeg + kchunk);
 
   float acc[NS][TM][TN];
-  small_tile_mainloop<NS, BM, BN, BK, TM, TN, PRO, VEC>(At, B, M, N, K, kbeg, kend, i0, j0, f, sm,
-                                                       acc);
+  small_tile_mainloop<NS, BM, BN, BK, TM, TN, PRO, VEC ? LD_WHOLE : LD_EACH>(
+      At, B, M, N, K, kbeg, kend, i0, j0, f, sm, acc);
   // partial tile to shared memory, then sum over the cluster's K ranges
 #pragma unroll
   for (int k = 0; k < NS; ++k)
@@ -553,13 +583,8 @@ k_group_small(const GroupProb* __restrict__ probs, const int2* __restrict__ work
   const int tn = (N + BN - 1) / BN;
   const int i0 = (w.y / tn) * BM, j0 = (w.y % tn) * BN;
   float acc[NS][TM][TN];
-  const float* At = o.fwd ? P.AhT : P.Ah;
-  const bool vec = (M | N) % 4 == 0 &&  // uniform over the problem's CTAs
-                   ((reinterpret_cast<uintptr_t>(At) | reinterpret_cast<uintptr_t>(o.B)) & 15) == 0;
-  if (vec)
-    small_tile_mainloop<NS, BM, BN, BK, TM, TN, true, true>(At, o.B, M, N, K, 0, K, i0, j0, f, sm, acc);
-  else
-    small_tile_mainloop<NS, BM, BN, BK, TM, TN, true, false>(At, o.B, M, N, K, 0, K, i0, j0, f, sm, acc);
+  small_tile_mainloop<NS, BM, BN, BK, TM, TN, true, LD_BRANCH>(o.fwd ? P.AhT : P.Ah, o.B, M, N, K, 0,
+                                                               K, i0, j0, f, sm, acc);
   coef_compute(o.coef, sh_coef);
   __syncthreads();
   const Out out{o.C, o.prev, nullptr, true, false, M, N, sh_coef[0], sh_coef[1]};
