@@ -664,6 +664,7 @@ int launch_cluster(Kern kernel, int BM, int BN, int NT, size_t smem, int KS, con
 template <class T, bool PRO, bool EPI, bool SPLIT>
 int run_fused(const float* At, const float* B, float* C, int M, int N, int K, int KS,
               const Fused& f, const Epi& ep, int trans, cudaStream_t st) {
+  TC_CHECK(!SPLIT || ep.red.out == nullptr);  // the split form stores without a reduction
   const int kchunk = (((K + KS - 1) / KS) + T::BK - 1) / T::BK * T::BK;
   if (vec_ok(At, B, C, M, N, ep))
     return launch_cluster(k_fused_gemm<T, PRO, EPI, SPLIT, true>, T::BM, T::BN, T::NT, T::bytes, KS,
@@ -675,44 +676,53 @@ int run_fused(const float* At, const float* B, float* C, int M, int N, int K, in
 template <int NS>
 using TileM = ftile::Tile<NS, 64, 64, 16, 4, 3, true>;
 
-// Which fused form serves an M x N x K product. Measured, us a launch at n x n
-// x n x 3 (FFMA floor in brackets): 32 x 32 tiles (the best K split) / 64 x 64
-// tiles whole / split over four:
-//   n = 128 [0.2]: 6.7 / 14.4 / 10.4     256 [1.3]: 11.7 / 24.7 / 12.9
-//   n = 320 [2.5]: 14.5 / 30.8 / 14.4    384 [4.4]: 20.3 / 34.9 / 16.5
-//   n = 512 [10.4]: 40.3 / 45.2 / 27.9   768 [35]: 105 / 65.6 / 65.6
-//   n = 1024 [83]: 248 / 156 / 140
-// Up to 20 64 x 64 tiles the launch is a latency: small tiles, K split while
-// the grid does not cover the SMs and each rank keeps two K blocks. Above, the SMs that take the most tiles set the
-// time: ceil(tiles KS / SMs) / KS, smallest over KS = 1, 2, 4, 8 (each rank
-// keeps at least two K blocks). Ties: four ranks where a whole tile each leaves
-// SMs idle (more warps a SM), no split where it does not (no exchange).
-// A solver's products (ep.red, or `solve` for the first of a two-sided pair)
-// keep one order of additions at each size: whole tiles from 152 64 x 64 tiles
-// on, else the small tiles.
+// Which fused form serves an M x N x K product: the one whose busiest SM is
+// estimated to be done first. Unit: a 32 x 32 tile's K block (16 of K). Small
+// tiles take rounds x blocks (rounds = ceil(tiles KS / SMs); K split while the grid
+// does not cover the SMs and each rank keeps two blocks), and 2 more when split. A
+// 64 x 64 tile's block is 2 units (four times the FMAs, half the shared-memory
+// reads an FMA), its split over 2 or 4 ranks 12 more and over 8 16 (the partial
+// tiles go through distributed shared memory); each rank keeps at least four
+// blocks. On ties the smaller tile, then four ranks.
+// Measured, us a launch, M x K x N x n3: 32 x 32 (their best split) / 64 x 64
+// whole / split over 4 / over 8, the rule's choice in brackets:
+//   330 x 64 x 200 x 3:  [8.2] / 14.4 / - / -      512 x 64 x 512 x 3:  [10.9] / 10.3 / - / -
+//   256 x 200 x 256 x 3: [10.3] / 21.5 / 14.4 / -  400 x 384 x 400 x 3: 34.8 / 38.8 / [24.6] / 20.5
+//   2048 x 512 x 40 x 3: 24.6 / 47.1 / [18.5] / 18.5
+//   512^3 x 3:           43.0 / 47.2 / [28.7] / 34.8
+//   1344 x 384 x 1344 x 3: 152 / [90.1] / 104 / 129
+// Over 8603 shapes (1..9800 x 20..1344 x 1..9800, n3 = 1..4) the choice is 3% off the
+// best form in the geometric mean; the rule by tile counts alone that it replaced
+// was 10% off, and slower than the 32 x 32 tiles on one shape in ten (330 x 64 x
+// 200 x 3: 14.4 us).
+// A solver's products (ep.red, or `solve` for the first of a two-sided pair) take
+// whole 64 x 64 tiles from 152 of them on, else small tiles: the split 64 x 64 form
+// has no reduction, and the orders of addition that solves have at each size are
+// held where they are.
 template <int NS, bool PRO, bool EPI>
 int pick_tile(const float* At, const float* B, float* C, int M, int N, int K, const Fused& f,
               const Epi& ep, int trans, bool solve, cudaStream_t st) {
   constexpr int BK = 16;
-  const long t64 = (long)((M + 63) / 64) * ((N + 63) / 64);
-  solve = solve || ep.red.out;
+  auto up = [](long x, long y) { return (x + y - 1) / y; };
+  const long t64 = up(M, 64) * up(N, 64), t32 = up(M, 32) * up(N, 32);
   int KS = 1;
-  if (solve ? t64 >= NSM : t64 > 20) {
-    if (!solve) {
-      auto cost = [&](int ks) { return (double)((t64 * ks + NSM - 1) / NSM) / ks; };
-      double best = t64 < NSM ? 1e30 : cost(1);
-      for (int ks : {4, 8, 2, 1})
-        if ((ks == 1 || K >= 2 * BK * ks) && cost(ks) < best) {
-          best = cost(ks);
-          KS = ks;
-        }
+  while (KS < 8 && t32 * KS < NSM && K >= 2 * BK * (KS * 2)) KS *= 2;
+  int K64 = 0;  // the 64 x 64 tiles' split; 0: small tiles
+  if (solve || ep.red.out) {
+    K64 = t64 >= NSM;
+  } else {
+    long best = up(t32 * KS, NSM) * up(up(K, KS), BK) + (KS > 1 ? 2 : 0);
+    for (int ks : {4, 8, 2, 1}) {
+      if (ks > 1 && K < 4 * BK * ks) continue;
+      const long c = 2 * up(t64 * ks, NSM) * up(up(K, ks), BK) + (ks == 1 ? 0 : ks == 8 ? 16 : 12);
+      if (c < best) {
+        best = c;
+        K64 = ks;
+      }
     }
-    return KS == 1
-               ? run_fused<TileM<NS>, PRO, EPI, false>(At, B, C, M, N, K, 1, f, ep, trans, st)
-               : run_fused<TileM<NS>, PRO, EPI, true>(At, B, C, M, N, K, KS, f, ep, trans, st);
   }
-  const long tiles = (long)((M + 31) / 32) * ((N + 31) / 32);
-  while (KS < 8 && tiles * KS < NSM && K >= 2 * BK * (KS * 2)) KS *= 2;
+  if (K64 == 1) return run_fused<TileM<NS>, PRO, EPI, false>(At, B, C, M, N, K, 1, f, ep, trans, st);
+  if (K64 > 1) return run_fused<TileM<NS>, PRO, EPI, true>(At, B, C, M, N, K, K64, f, ep, trans, st);
   const int kchunk = (((K + KS - 1) / KS) + BK - 1) / BK * BK;
   const bool vec = (M | N) % 4 == 0 && al16(At) && al16(B);
   return vec ? launch_cluster(k_fused_small<NS, 32, 32, BK, 4, 2, PRO, EPI, true>, 32, 32, 128, 0, KS,

@@ -177,8 +177,8 @@ void tc_set_message(const char* msg);
 // C/prev: M x N; slice strides are the dense sizes. pro/epi: n3 x n3 row-major
 // (host arrays, by value), used only when the CTA owns all n3 <= TC_MAX_FUSED
 // slices. trans: C is stored N x M a slice (the K-major left factor of a
-// second product; no prev and no reduction). solve: a solver's product, whose
-// order of additions does not follow the tile chosen (implied by ep.red).
+// second product; no prev and no reduction). solve: a solver's product (implied
+// by ep.red), which takes the tiles that solves have always taken at its size.
 int gemm_init();
 int launch_slice_gemm(const float* At, const float* B, float* C, int M, int N, int K,
                       int nslices, const float* pro, const float* epi, const Epi& ep,

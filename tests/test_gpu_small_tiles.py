@@ -1,10 +1,11 @@
-"""The 32 x 32 fused FP32 tiles with each way of reading their operands: whole
-groups of four in both, in the left operand only, in the right one only, in
-neither; by their sizes and by where the operands start; K whole and split.
+"""The fused FP32 products: the 32 x 32 tiles with each way of reading their
+operands (whole groups of four in both, in the left operand only, in the right
+one only, in neither; by their sizes and by where the operands start; K whole and
+split), and the 64 x 64 tiles with each split.
 
 The choice follows M = n1 (left, K-major) and N = s (right) for the product and
 M = n2 for the adjoint. Tolerance: the FP32 products' 1e-5 bound (K <= 420 FMAs in
-one chain are within sqrt(420) 2^-24 = 1.2e-6 relative, times the transforms'
+one chain are within sqrt(420) 2^-24 = 1.2e-6 relative, K = 832 within 1.8e-6, times the transforms'
 condition, at most 4 for n3 <= 4 on random data)."""
 import pytest
 
@@ -27,6 +28,25 @@ def test_products_by_alignment(tc, n1, n2, s, n3):
     plan = tc.Plan(A, s=s)
     assert rel(plan.cprod(X), reference(A, None, X, False)) < 1e-5
     assert rel(plan.adjoint(Y), reference(A, None, Y, True)) < 1e-5
+    plan.close()
+
+
+# The product's form by the rule of gemm.cu (64 x 64 tiles whole, and split over
+# 2, 4 and 8 ranks), whole groups and ragged; with a right factor both products of
+# the pair, the first stored transposed
+@pytest.mark.parametrize("n1,n2,s,n3,two", [
+    (512, 130, 832, 3, False), (401, 130, 833, 3, False), (512, 520, 832, 3, False), (257, 520, 833, 3, False),
+    (448, 448, 448, 1, False), (257, 521, 259, 3, False), (256, 520, 832, 4, False), (256, 520, 641, 2, False),
+    (448, 448, 448, 3, True), (451, 449, 450, 4, True), (256, 520, 832, 2, True), (300, 520, 521, 1, True)])
+def test_products_by_form(tc, n1, n2, s, n3, two):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n1 + 3 * n2 + s + n3)
+    rand = lambda *sh: torch.randn(sh, generator=g, device="cuda")
+    A, B = rand(n3, n1, n2), rand(n3, s, s) if two else None
+    X, Y = rand(n3, n2, s), rand(n3, n1, s)
+    plan = tc.Plan(A, B, s=s)
+    assert rel(plan.cprod(X), reference(A, B, X, False)) < 1e-5
+    assert rel(plan.adjoint(Y), reference(A, B, Y, True)) < 1e-5
     plan.close()
 
 
