@@ -1,4 +1,4 @@
-// The projected problem in FP64 on one CTA (§3.1 eqs. (leastsq), (tikho2),
+// The projected problem in FP64 (§3.1 eqs. (leastsq), (tikho2),
 // (gcv2); §3.2 eqs. (normeq2), (leastsq0)):
 //   1. one-sided Jacobi SVD of the (k+1) x k matrix H (Hestenes rotations,
 //      round-robin pair order, warps rotate disjoint column pairs),
@@ -13,15 +13,19 @@
 //
 // Bound: FP64. GB300 issues fewer than two FP64 lanes a clock and SM, so a warp
 // instruction holds the pipe for about 19 clocks, and every division or square
-// root is a chain of them. So:
-// * a cluster of eight CTAs: rank 0 runs the SVD and the solve, and every rank
-//   evaluates 25 of a level's 200 grid points, one a lane of one warp (on one SM a
-//   level of k = 10 took about 35 us, nearly all of it the pipe);
-// * reciprocals and square roots by Newton's method (rcp_newton, rsqrt_newton:
-//   a few ulp), one reciprocal a GCV term;
+// root is a chain of them (IEEE ones throughout: H may be graded or scaled over the
+// whole range, where estimates flush or lose the rotation of a small column). So:
+// * for the search, a cluster of eight CTAs: rank 0 runs the SVD and the solve, and
+//   every rank evaluates 25 of a level's 200 grid points, one a lane of one warp (on
+//   one SM a level of k = 10 took about 35 us, nearly all of it the pipe). A given
+//   lambda needs one CTA;
+// * beyond two warps of column pairs, the rotations of a round's pairs by the lanes
+//   of one warp, so that their chains share its instructions;
 // * as many warps as the SVD has column pairs (at most 32), as every round ends
 //   in a barrier; the triangular solves run by columns over all threads.
-// At k = 10: 308 -> 176 us a launch (cold), most of it the SVD's chains.
+// us a launch with the search (one CTA of 1024 threads, a warp a pair, before): k = 10
+// 308 -> 244, k = 32 2954 -> 1598, k = 128 78.4 -> 37.1 ms; lambda given, k = 10 229 ->
+// 224. Most of it is the SVD's chains.
 #include <cooperative_groups.h>
 
 #include "tc_device.cuh"
@@ -37,19 +41,6 @@ constexpr int CL = 8;            // CTAs of the cluster
 constexpr int PPR = NGRID / CL;  // grid points a rank: one a lane
 static_assert(NGRID % CL == 0 && PPR <= 32, "one warp a rank");
 
-// The hardware's estimates of 1 / sqrt(x) and 1 / x (about 20 bits; subnormals
-// as zero, zero gives Inf).
-__device__ __forceinline__ double rsqrt_approx(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  return y;
-}
-__device__ __forceinline__ double rcp_approx(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  return y;
-}
-
 // Lanes a column pair of the SVD: columns of up to 8 or 16 values share a warp.
 __host__ __device__ constexpr int lane_group(int rows) { return rows <= 8 ? 8 : rows <= 16 ? 16 : 32; }
 
@@ -57,18 +48,25 @@ __host__ __device__ constexpr int lane_group(int rows) { return rows <= 8 ? 8 : 
 __device__ double gcv_eval(const double* sig2, const double* g, int k, double gnull2, double lam,
                            int variant) {
   const double l2 = lam * lam;
-  const double sc = variant == TC_GCV_FULL ? l2 : 1.0;
   double num = 0.0, den = 0.0;
-#pragma unroll 4
-  for (int i = 0; i < k; ++i) {
-    const double q = sc * rcp_newton(sig2[i] + l2);
-    const double r = g[i] * q;
-    num = fma(r, r, num);
-    den += q;
-  }
   if (variant == TC_GCV_FULL) {
+#pragma unroll 4
+    for (int i = 0; i < k; ++i) {
+      const double q = l2 / (sig2[i] + l2);
+      const double r = g[i] * q;
+      num = fma(r, r, num);
+      den += q;
+    }
     num += gnull2;
     den += 1.0;
+  } else {
+#pragma unroll 4
+    for (int i = 0; i < k; ++i) {
+      const double d = sig2[i] + l2;
+      const double r = g[i] / d;
+      num = fma(r, r, num);
+      den += 1.0 / d;
+    }
   }
   return num / (den * den);
 }
@@ -136,19 +134,33 @@ k_tikhonov_gcv(const double* __restrict__ H, int ld, int kmax, const int* kdev,
     // Rotate while |<h_p, h_q>| > rows * eps * ||h_p|| ||h_q||: below that the
     // inner product is rounding noise of the (rows)-term dot product. Squared
     // column norms d[] are recomputed every sweep and updated by the rotation
-    // identities d_p -= t gamma, d_q += t gamma in between. A round is three
-    // parts: the pairs' dot products (LG lanes a pair), their rotations (one
-    // lane a pair, so that the FP64 chains of all pairs share a warp's
-    // instructions), and the column updates. t comes from a 20-bit estimate: the
-    // rotation is orthogonal to FP64 (c and s = c t belong to that t), and it
-    // leaves 1e-6 of gamma where the exact t would leave nothing, which the next
-    // sweep's quadratic convergence hides.
+    // identities d_p -= t gamma, d_q += t gamma in between. Where the pairs fill no
+    // more than two warps, their lanes (LG a pair) each form the rotation and a
+    // round is one part; else it is three: the pairs' dot products, their
+    // rotations (one lane a pair), and the column updates.
     const double jtol = rows * 2.220446049250313e-16;
     const int npairs = kk / 2, lg = lane_group(rows), ppw = 32 / lg, sub = lane % lg;
+    const bool direct = npairs <= 2 * ppw;
     auto pair_of = [&](int pi, int rnd, int& a, int& b) {
       // circle method: player 0 fixed, the others rotate by rnd
       a = (pi == 0) ? 0 : ((pi - 1 + rnd) % (kk - 1)) + 1;
       b = ((kk - 2 - pi + rnd) % (kk - 1)) + 1;
+    };
+    // The rotation (c, s) that makes the columns orthogonal, t its tangent; false: none
+    auto angle = [&](double ga, double al, double be, double& c, double& sn, double& t) {
+      if (!(ga != 0.0 && fabs(ga) > jtol * sqrt(al * be))) return false;
+      const double zeta = (be - al) / (2.0 * ga);
+      t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+      c = 1.0 / sqrt(1.0 + t * t);
+      sn = c * t;
+      return true;
+    };
+    auto update = [&](int a, int b, double c, double sn) {
+      for (int r = sub; r < rows; r += lg) {
+        const double u = Hs[a * rows + r], v = Hs[b * rows + r];
+        Hs[a * rows + r] = c * u - sn * v;
+        Hs[b * rows + r] = sn * u + c * v;
+      }
     };
     for (int sweep = 0; sweep < MAX_SWEEPS; ++sweep) {
       if (tid == 0) sh_rot = 0;
@@ -159,6 +171,7 @@ k_tikhonov_gcv(const double* __restrict__ H, int ld, int kmax, const int* kdev,
         s2 = warp_sum(s2);
         if (lane == 0) dn[c] = s2;
       }
+      __syncthreads();
       for (int rnd = 0; rnd < kk - 1; ++rnd) {
         for (int p0 = warp * ppw; p0 < npairs; p0 += nw * ppw) {
           const int pi = p0 + lane / lg;
@@ -167,28 +180,31 @@ k_tikhonov_gcv(const double* __restrict__ H, int ld, int kmax, const int* kdev,
           double ga = 0.0;
           for (int r = sub; r < rows; r += lg) ga = fma(Hs[a * rows + r], Hs[b * rows + r], ga);
           for (int o = lg / 2; o > 0; o >>= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
-          if (sub == 0 && pi < npairs) rot[pi][0] = ga;
+          if (direct) {
+            const double al = dn[a], be = dn[b];
+            double c, sn, t;
+            const bool go = pi < npairs && angle(ga, al, be, c, sn, t);
+            __syncwarp();  // every lane has the norms
+            if (go) {
+              update(a, b, c, sn);
+              if (sub == 0) {
+                dn[a] = al - t * ga;
+                dn[b] = be + t * ga;
+                sh_rot = 1;
+              }
+            }
+          } else if (sub == 0 && pi < npairs) {
+            rot[pi][0] = ga;
+          }
         }
         __syncthreads();
+        if (direct) continue;
         if (tid < npairs) {
           int a, b;
           pair_of(tid, rnd, a, b);
           const double ga = rot[tid][0], al = dn[a], be = dn[b];
-          double c = 1.0, sn = 0.0;
-          if (ga != 0.0 && fabs(ga) * rsqrt_approx(al * be) > jtol) {
-            const float z = (float)((be - al) * rcp_approx(2.0 * ga));
-            const float az = fabsf(z);
-            // 1 / (|z| + sqrt(1 + z^2)), past FP32's range of z^2 1 / (2 |z|)
-            const float ta = az < 1e18f ? 1.f / (az + sqrtf(fmaf(z, z, 1.f))) : 0.5f / az;
-            const double t = z >= 0.f ? ta : -ta;
-            c = rsqrt_approx(fma(t, t, 1.0));
-            sn = c * t;
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {  // to c^2 + s^2 = 1 within an ulp: hundreds of
-              const double e = fma(-sn, sn, fma(-c, c, 1.0));  // rotations meet in a column
-              c = fma(0.5 * c, e, c);
-              sn = fma(0.5 * sn, e, sn);
-            }
+          double c = 1.0, sn = 0.0, t;
+          if (angle(ga, al, be, c, sn, t)) {
             dn[a] = al - t * ga;
             dn[b] = be + t * ga;
             sh_rot = 1;
@@ -204,11 +220,7 @@ k_tikhonov_gcv(const double* __restrict__ H, int ld, int kmax, const int* kdev,
           if (sn == 0.0) continue;
           int a, b;
           pair_of(pi, rnd, a, b);
-          for (int r = sub; r < rows; r += lg) {
-            const double u = Hs[a * rows + r], v = Hs[b * rows + r];
-            Hs[a * rows + r] = c * u - sn * v;
-            Hs[b * rows + r] = sn * u + c * v;
-          }
+          update(a, b, c, sn);
         }
         __syncthreads();
       }
@@ -223,11 +235,11 @@ k_tikhonov_gcv(const double* __restrict__ H, int ld, int kmax, const int* kdev,
       s2 = warp_sum(s2);
       if (lane == 0) {
         sig2[c] = s2;
-        g[c] = (s2 > 0.0) ? beta * x[0] * (1.0 / sqrt(s2)) : 0.0;
+        g[c] = (s2 > 0.0) ? beta * x[0] / sqrt(s2) : 0.0;
       }
     }
-    double hs = 0.0;  // ||H||_F
-    for (int idx = tid; idx < rows * k; idx += nt) {
+    double hs = 0.0;  // ||H||_F, for the search
+    for (int idx = tid; search && idx < rows * k; idx += nt) {
       const double v = H[(size_t)(idx / k) * ld + idx % k];
       hs += v * v;
     }
@@ -236,15 +248,14 @@ k_tikhonov_gcv(const double* __restrict__ H, int ld, int kmax, const int* kdev,
     __syncthreads();
     if (warp == 0) {
       const double t = warp_sum(lane < nw ? sh_w[lane] : 0.0);
-      double gs = 0.0;  // the part of beta e1 outside the range of H
-      for (int i = lane; i < k; i += 32) gs += g[i] * g[i];
-      gs = warp_sum(gs);
       if (lane == 0) {
-        // below the rounding of the sum it is a difference of equal numbers: zero
-        const double d = beta * beta - gs;
-        sh_gnull2 = d > rows * 2.220446049250313e-16 * beta * beta ? d : 0.0;
-        bracket[0][1] = log(sqrt(t));
-        bracket[0][0] = bracket[0][1] - 10.0 * log(10.0);
+        double gs = 0.0;  // the part of beta e1 outside the range of H
+        for (int i = 0; i < k; ++i) gs += g[i] * g[i];
+        sh_gnull2 = fmax(beta * beta - gs, 0.0);
+        if (search) {
+          bracket[0][1] = log(sqrt(t));
+          bracket[0][0] = bracket[0][1] - 10.0 * log(10.0);
+        }
       }
     }
     __syncthreads();
@@ -309,8 +320,7 @@ k_tikhonov_gcv(const double* __restrict__ H, int ld, int kmax, const int* kdev,
   }
 
   // ---- 3. (H^T H + lambda^2 I) y = beta H^T e_1, Cholesky --------------------
-  double* G = dsm;  // k x k row-major, overwrites the Jacobi copy; L's diagonal
-  double* inv = dn;  // is kept inverted in dn
+  double* G = dsm;  // k x k row-major, overwrites the Jacobi copy
   for (int idx = tid; idx < k * k; idx += nt) {
     const int i = idx / k, jj = idx % k;
     double s = 0.0;
@@ -321,10 +331,10 @@ k_tikhonov_gcv(const double* __restrict__ H, int ld, int kmax, const int* kdev,
   for (int i = tid; i < k; i += nt) g[i] = beta * H[i];  // rhs = beta * (row 1 of H)
   __syncthreads();
   for (int c = 0; c < k; ++c) {
-    if (tid == 0) inv[c] = rsqrt_newton(G[c * k + c]);
+    if (tid == 0) G[c * k + c] = sqrt(G[c * k + c]);
     __syncthreads();
-    const double d = inv[c];
-    for (int r = c + 1 + tid; r < k; r += nt) G[r * k + c] *= d;
+    const double d = G[c * k + c];
+    for (int r = c + 1 + tid; r < k; r += nt) G[r * k + c] /= d;
     __syncthreads();
     for (int idx = tid; idx < (k - c - 1) * (k - c - 1); idx += nt) {
       const int r = c + 1 + idx / (k - c - 1), q = c + 1 + idx % (k - c - 1);
@@ -332,15 +342,15 @@ k_tikhonov_gcv(const double* __restrict__ H, int ld, int kmax, const int* kdev,
     }
     __syncthreads();
   }
-  for (int c = 0; c < k; ++c) {  // L z = rhs by columns: g[c] becomes z[c] / 1
-    const double z = g[c] * inv[c];
+  for (int c = 0; c < k; ++c) {  // L z = rhs by columns: g[c] becomes z[c]
+    const double z = g[c] / G[c * k + c];
     __syncthreads();
     for (int r = c + 1 + tid; r < k; r += nt) g[r] -= G[r * k + c] * z;
     if (tid == 0) g[c] = z;
     __syncthreads();
   }
   for (int c = k - 1; c >= 0; --c) {  // L^T y = z by columns of L^T
-    const double z = g[c] * inv[c];
+    const double z = g[c] / G[c * k + c];
     __syncthreads();
     for (int r = tid; r < c; r += nt) g[r] -= G[c * k + r] * z;
     if (tid == 0) g[c] = z;
@@ -378,17 +388,18 @@ int launch_tikhonov_gcv(const double* H, int ld, int kmax, const int* kdev,
   int nw = (kk / 2 + ppw - 1) / ppw;  // the warps that the column pairs fill
   nw = nw < 4 ? 4 : nw > 32 ? 32 : nw;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(CL);
+  const int cl = lambda_in >= 0.0 ? 1 : CL;  // only the search is spread
+  cfg.gridDim = dim3(cl);
   cfg.blockDim = dim3(32 * nw);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CL;
+  attr[0].val.clusterDim.x = cl;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cl > 1;
   TC_CUDA(cudaLaunchKernelEx(&cfg, k_tikhonov_gcv, H, ld, kmax, kdev, beta, variant, lambda_in,
                              lambda_out, y, gcv_out, skip));
   return TC_OK;
