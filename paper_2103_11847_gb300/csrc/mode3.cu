@@ -15,7 +15,10 @@
 //   block's results are stored. (Requesting a block as a whole once the last
 //   one's FMAs were done left the FMA pipe 52% busy: 73 us at n3 = 64.)
 // * prev is read four rows ahead of the stores (it may alias out, so the
-//   compiler cannot move a read over an earlier store by itself).
+//   compiler cannot move a read over an earlier store by itself); up to n3 = 16,
+//   where a CTA has one block, the first rows before the FMAs: nothing else of
+//   such a launch overlaps the read (144 x 144 x 9 c-LSQR with BF16X3 products, 6
+//   steps: 318 us without it, 310 with).
 // TRANS (TF32 operand of the tensor-core GEMM, which reads it K-major): a block
 // is 8 rows x 16 columns of the K x N pixel grid and is stored N x K a slice, 32
 // contiguous bytes a column, in place of a separate transposition pass.
@@ -78,6 +81,9 @@ __global__ void __launch_bounds__(NT, KPW == 8 ? 3 : (KPW == 4 ? 5 : (KPW == 2 ?
 k_mode3(const float* __restrict__ in, void* out_v, const float* __restrict__ Tt, int n3, size_t P,
         size_t nblk, Grid2 g, Epi ep) {
   constexpr int NK = 8 * KPW, TK = 2 * KPW, SF = slice_floats<TRANS>(), LG = slot_rows<KPW>();
+  constexpr int G = TK < 4 ? TK : 4;  // rows of prev read ahead of their stores
+  constexpr bool EARLY = OUT == OUT_F32 && KPW <= 2;  // the first of them ahead of the FMAs
+  const bool alone = nblk <= gridDim.x;               // where a CTA has one block
   if (ep.skip && *ep.skip) return;
   extern __shared__ __align__(16) float m3_smem[];
   float(*ts)[NK] = reinterpret_cast<float(*)[NK]>(m3_smem);  // ts[l][k] = T[k][l]
@@ -145,6 +151,17 @@ k_mode3(const float* __restrict__ in, void* out_v, const float* __restrict__ Tt,
     for (int q = 0; q < KPW; ++q)
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[q][e] = 0ull;
+    float4 pv[G];
+    auto load_prev = [&](int q0, size_t pb, size_t idx0) {
+#pragma unroll
+      for (int q = 0; q < G; ++q)
+        if (VEC && ep.prev && pb < P && w * TK + q0 + q < n3)
+          pv[q] = *reinterpret_cast<const float4*>(ep.prev + idx0 + (q0 + q) * P);
+    };
+    if (EARLY && alone) {
+      const size_t p0 = blk * PB + lane * 4;
+      load_prev(0, p0, (size_t)(w * TK) * P + p0);
+    }
     for (int c = 0; c < nch; ++c) {
       ftile::cp_wait<S - 2>();  // this thread's copies of the slot have landed
       __syncthreads();  // everyone's (and T); every warp is done with the slot refilled now
@@ -247,16 +264,9 @@ k_mode3(const float* __restrict__ in, void* out_v, const float* __restrict__ Tt,
     const float ca = sh_coef[0], cp = sh_coef[1];
     const size_t idx0 = (size_t)(w * TK) * P + pb;
     float local[2] = {0.f, 0.f};  // of virtual warps 2w and 2w + 1
-    constexpr int G = TK < 4 ? TK : 4;  // rows of prev read ahead of their stores
 #pragma unroll
     for (int q0 = 0; q0 < TK; q0 += G) {
-      float4 pv[G];
-#pragma unroll
-      for (int q = 0; q < G; ++q) {
-        const int k = w * TK + q0 + q;
-        if (VEC && ep.prev && pb < P && k < n3)
-          pv[q] = *reinterpret_cast<const float4*>(ep.prev + idx0 + (q0 + q) * P);
-      }
+      if (!EARLY || !alone || q0 > 0) load_prev(q0, pb, idx0);
 #pragma unroll
       for (int q = 0; q < G; ++q) {
         const int k = w * TK + q0 + q;

@@ -155,14 +155,21 @@ template <int V>
 __device__ __forceinline__ void sum_partials(const Red& red, size_t nblk) {
   __shared__ double sh_d[4 * V];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  if (tid < 128) {
+  if (tid < 128) {  // the V chains of a thread side by side
+    double acc[V];
 #pragma unroll
-    for (int q = 0; q < V; ++q) {
-      double acc = 0.0;
-      for (size_t i = tid + 128 * q; i < nblk; i += 128 * V) acc += __ldcg(red.partials + i);
-      acc = warp_sum(acc);
-      if (lane == 0) sh_d[4 * q + w] = acc;
-    }
+    for (int q = 0; q < V; ++q) acc[q] = 0.0;
+    for (size_t i = tid; i < nblk; i += 128 * V)
+#pragma unroll
+      for (int q = 0; q < V; ++q)
+        if (i + 128 * q < nblk) acc[q] += __ldcg(red.partials + i + 128 * q);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int q = 0; q < V; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+    if (lane == 0)
+#pragma unroll
+      for (int q = 0; q < V; ++q) sh_d[4 * q + w] = acc[q];
   }
   __syncthreads();
   if (tid < 32) {
