@@ -33,7 +33,7 @@ __device__ __forceinline__ float gelu_d(float z) {
 }
 
 // The pass over samples, four a CTA of 256 threads (64 a sample): forward, and
-// with targets (T non-null) the loss and the backward pass through the
+// with targets (TRAIN) the loss and the backward pass through the
 // activations, D = (out - t) / B, dZ2 = (D W3^T) * gelu'(z2), dZ1 = (dZ2 W2^T) *
 // gelu'(z1).
 //
@@ -41,11 +41,16 @@ __device__ __forceinline__ float gelu_d(float z) {
 // of at most 64 FMAs). The BF16 weights are staged in shared memory once a CTA
 // with 16-byte copies; W2's rows are 66 values apart, so that both its columns
 // (forward) and its rows (backward) are read without bank conflicts. z1 and z2
-// stay in registers.
-constexpr int SPC = 4;           // samples a CTA
+// stay in registers. A forward pass of many samples takes the CTAs that fit, eight
+// a SM, each over several groups of four, so that the weights are staged once a CTA
+// and the next group's inputs are on their way (200000 samples 281 us; one group a
+// CTA 303, one sample a CTA reading the weights from L1 291; 20000: 32.8, 34.8, 32.8).
+constexpr int SPC = 4;           // samples a group
+constexpr int CTAS = 8;          // a SM
 constexpr int W2S = NH + 2;      // row stride of W2 in shared memory
 
-__global__ void __launch_bounds__(SPC * NH)
+template <bool TRAIN>  // with targets: one group a CTA
+__global__ void __launch_bounds__(SPC * NH, TRAIN ? 0 : CTAS)
 k_mlp_samples(const float* __restrict__ X, const float* __restrict__ T, int B,
               const __nv_bfloat16* Wb, const float* theta, float* H1, float* H2, float* OUT,
               float* D, float* dZ1, float* dZ2, float* lossb) {
@@ -54,12 +59,11 @@ k_mlp_samples(const float* __restrict__ X, const float* __restrict__ T, int B,
   __shared__ __align__(16) __nv_bfloat16 w3[NH * NO];
   __shared__ float xs[SPC][NI], h1s[SPC][NH], h2s[SPC][NH], dz2s[SPC][NH], ds[SPC][NO];
   const int tid = threadIdx.x, q = tid / NH, j = tid % NH;
-  const int b = blockIdx.x * SPC + q;
-  const bool live = b < B;
-  for (int i = tid; i < SPC * NI; i += SPC * NH) {
-    const int bb = blockIdx.x * SPC + i / NI;
-    xs[i / NI][i % NI] = bb < B ? X[(size_t)blockIdx.x * SPC * NI + i] : 0.f;
-  }
+  static_assert(SPC * NI <= SPC * NH, "an input a thread");
+  auto input = [&](int g) {  // thread tid's of group g's inputs
+    return tid < SPC * NI && g * SPC + tid / NI < B ? X[(size_t)g * SPC * NI + tid] : 0.f;
+  };
+  float x = input(blockIdx.x);
   pdl_trigger();
   pdl_wait();  // the weights are the last step's
   for (int i = tid; i < NI * NH / 8; i += SPC * NH)
@@ -71,52 +75,60 @@ k_mlp_samples(const float* __restrict__ X, const float* __restrict__ T, int B,
   }
   if (tid < NH * NO / 8) reinterpret_cast<uint4*>(w3)[tid] = reinterpret_cast<const uint4*>(Wb + OW3)[tid];
   const float bias1 = theta[OB1 + j], bias2 = theta[OB2 + j];
-  __syncthreads();
-  float z1 = bias1;
+  const int groups = (B - 1) / SPC + 1;
+  for (int grp = blockIdx.x; grp < groups; grp += gridDim.x) {
+    const int b = grp * SPC + q;
+    const bool live = b < B;
+    if (tid < SPC * NI) xs[tid / NI][tid % NI] = x;  // the last group's have been used
+    __syncthreads();
+    if (!TRAIN && grp + (int)gridDim.x < groups) x = input(grp + gridDim.x);
+    float z1 = bias1;
 #pragma unroll
-  for (int i = 0; i < NI; ++i) z1 = fmaf(xs[q][i], __bfloat162float(w1[i * NH + j]), z1);
-  const float h1 = gelu(z1);
-  h1s[q][j] = h1;
-  if (H1 && live) H1[(size_t)b * NH + j] = h1;
-  __syncthreads();
-  float z2 = bias2;
+    for (int i = 0; i < NI; ++i) z1 = fmaf(xs[q][i], __bfloat162float(w1[i * NH + j]), z1);
+    const float h1 = gelu(z1);
+    h1s[q][j] = h1;
+    if (H1 && live) H1[(size_t)b * NH + j] = h1;
+    __syncthreads();
+    float z2 = bias2;
 #pragma unroll
-  for (int i = 0; i < NH; ++i) z2 = fmaf(h1s[q][i], __bfloat162float(w2[i * W2S + j]), z2);
-  const float h2 = gelu(z2);
-  h2s[q][j] = h2;
-  if (H2 && live) H2[(size_t)b * NH + j] = h2;
-  __syncthreads();
-  if (j < NO) {
-    float o = theta[OB3 + j];
+    for (int i = 0; i < NH; ++i) z2 = fmaf(h1s[q][i], __bfloat162float(w2[i * W2S + j]), z2);
+    const float h2 = gelu(z2);
+    h2s[q][j] = h2;
+    if (H2 && live) H2[(size_t)b * NH + j] = h2;
+    __syncthreads();
+    if (j < NO) {
+      float o = theta[OB3 + j];
 #pragma unroll
-    for (int i = 0; i < NH; ++i) o = fmaf(h2s[q][i], __bfloat162float(w3[i * NO + j]), o);
-    if (OUT && live) OUT[(size_t)b * NO + j] = o;
-    if (T) {
-      const float r = live ? o - T[(size_t)b * NO + j] : 0.f;
-      ds[q][j] = r / B;
-      if (live) D[(size_t)b * NO + j] = r / B;
-      float l = 0.f;  // threads 0 and 1 of the sample are neighbours in one warp
+      for (int i = 0; i < NH; ++i) o = fmaf(h2s[q][i], __bfloat162float(w3[i * NO + j]), o);
+      if (OUT && live) OUT[(size_t)b * NO + j] = o;
+      if (TRAIN) {
+        const float r = live ? o - T[(size_t)b * NO + j] : 0.f;
+        ds[q][j] = r / B;
+        if (live) D[(size_t)b * NO + j] = r / B;
+        float l = 0.f;  // threads 0 and 1 of the sample are neighbours in one warp
 #pragma unroll
-      for (int k = 0; k < NO; ++k) {
-        const float rk = __shfl_sync((1u << NO) - 1, r, k, NO);
-        l = fmaf(rk, rk, l);
+        for (int k = 0; k < NO; ++k) {
+          const float rk = __shfl_sync((1u << NO) - 1, r, k, NO);
+          l = fmaf(rk, rk, l);
+        }
+        if (j == 0 && live) lossb[b] = 0.5f * l / B;
       }
-      if (j == 0 && live) lossb[b] = 0.5f * l / B;
     }
+    if (!TRAIN) continue;
+    __syncthreads();
+    float g = 0.f;
+#pragma unroll
+    for (int o = 0; o < NO; ++o) g = fmaf(ds[q][o], __bfloat162float(w3[j * NO + o]), g);
+    const float dz2 = g * gelu_d(z2);
+    dz2s[q][j] = dz2;
+    if (live) dZ2[(size_t)b * NH + j] = dz2;
+    __syncthreads();
+    g = 0.f;
+#pragma unroll
+    for (int k = 0; k < NH; ++k) g = fmaf(dz2s[q][k], __bfloat162float(w2[j * W2S + k]), g);
+    if (live) dZ1[(size_t)b * NH + j] = g * gelu_d(z1);
+    return;
   }
-  if (!T) return;
-  __syncthreads();
-  float g = 0.f;
-#pragma unroll
-  for (int o = 0; o < NO; ++o) g = fmaf(ds[q][o], __bfloat162float(w3[j * NO + o]), g);
-  const float dz2 = g * gelu_d(z2);
-  dz2s[q][j] = dz2;
-  if (live) dZ2[(size_t)b * NH + j] = dz2;
-  __syncthreads();
-  g = 0.f;
-#pragma unroll
-  for (int k = 0; k < NH; ++k) g = fmaf(dz2s[q][k], __bfloat162float(w2[j * W2S + k]), g);
-  if (live) dZ1[(size_t)b * NH + j] = g * gelu_d(z1);
 }
 
 // Adam (bias-corrected) on parameter p; refreshes its BF16 copy.
@@ -400,7 +412,7 @@ int fwd_bwd(tc_mlp* m, const float* X, const float* T, int B, float* grad, float
   float* dZ1 = D + (size_t)kMaxB * NO;
   float* dZ2 = dZ1 + (size_t)kMaxB * NH;
   float* lossb = dZ2 + (size_t)kMaxB * NH;
-  TC_TRY(launch_pdl(!first, k_mlp_samples, (B + SPC - 1) / SPC, SPC * NH, st, X, T, B, m->Wb, m->theta, H1,
+  TC_TRY(launch_pdl(!first, k_mlp_samples<true>, (B + SPC - 1) / SPC, SPC * NH, st, X, T, B, m->Wb, m->theta, H1,
                     H2, (float*)nullptr, D, dZ1, dZ2, lossb));
   return launch_pdl(true, k_mlp_grad, GCTAS, GT, st, X, B, H1, H2, D, dZ1, dZ2, lossb, grad, loss, a);
 }
@@ -415,7 +427,8 @@ extern "C" int tc_mlp_loss_grad(tc_mlp* m, const float* X, const float* T, int B
 extern "C" int tc_mlp_forward(tc_mlp* m, const float* X, int B, float* Y, tc_stream_t stream) {
   if (!m || !X || !Y || B < 1) return TC_EINVAL;
   float* none = nullptr;
-  return launch_pdl(false, k_mlp_samples, (B + SPC - 1) / SPC, SPC * NH, (cudaStream_t)stream, X,
+  const int groups = (B - 1) / SPC + 1, fit = 152 * CTAS;
+  return launch_pdl(false, k_mlp_samples<false>, groups < fit ? groups : fit, SPC * NH, (cudaStream_t)stream, X,
                     none, B, m->Wb, m->theta, none, none, Y, none, none, none, none);
 }
 
