@@ -3,6 +3,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -605,11 +606,17 @@ extern "C" int tc_plan_create(tc_plan** out, int n1, int n2, int s, int n3, cons
     // TMA), the transform passes of the unfused route
     if (n1 % 8 || n2 % 8 || s % 8) return TC_EUNSUPPORTED;
   }
-  static int inited = 0;
-  if (!inited) {
-    TC_TRY(tc_kernels_init());
-    TC_TRY(umma_init());
-    inited = 1;
+  {  // kernel attributes (shared memory beyond 48 KB) are a device's own
+    static std::mutex mu;
+    static bool inited[64];
+    int dev = 0;
+    TC_CUDA(cudaGetDevice(&dev));
+    const std::lock_guard<std::mutex> lock(mu);
+    if (dev >= 64 || !inited[dev]) {
+      TC_TRY(tc_kernels_init());
+      TC_TRY(umma_init());
+      if (dev < 64) inited[dev] = true;
+    }
   }
   tc_plan* p = new (std::nothrow) tc_plan();
   if (!p) return TC_ENOMEM;

@@ -412,8 +412,8 @@ int launch_build_bidiag(const double* alpha, const double* beta, const int* kdev
   return TC_OK;
 }
 
-// Called once per process (from plan creation) so that no attribute call
-// happens while a stream is being captured.
+// Called once a device (from plan creation) so that no attribute call happens
+// while a stream is being captured.
 int tc_kernels_init() {
   TC_CUDA(cudaFuncSetAttribute(k_tikhonov_gcv, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                200 * 1024));

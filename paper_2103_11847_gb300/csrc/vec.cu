@@ -521,11 +521,12 @@ int vec_init() {
   TC_CUDA(cudaFuncSetAttribute(k_scale, cudaFuncAttributePreferredSharedMemoryCarveout, c));
   TC_CUDA(cudaFuncSetAttribute(k_lsqr_update<float>, cudaFuncAttributePreferredSharedMemoryCarveout, c));
   TC_CUDA(cudaFuncSetAttribute(k_lsqr_update<float4>, cudaFuncAttributePreferredSharedMemoryCarveout, c));
-  g_ao_ok = true;
-  TC_TRY(init_ao<1>(&g_ao_ok));
-  TC_TRY(init_ao<2>(&g_ao_ok));
-  TC_TRY(init_ao<3>(&g_ao_ok));
-  TC_TRY(init_ao<4>(&g_ao_ok));
+  bool ok = true;
+  TC_TRY(init_ao<1>(&ok));
+  TC_TRY(init_ao<2>(&ok));
+  TC_TRY(init_ao<3>(&ok));
+  TC_TRY(init_ao<4>(&ok));
+  g_ao_ok = ok;
   int dev = 0;
   TC_CUDA(cudaGetDevice(&dev));
   TC_CUDA(cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev));
