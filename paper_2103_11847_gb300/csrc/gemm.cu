@@ -456,7 +456,9 @@ k_fused_small(const float* __restrict__ At, const float* __restrict__ B, float* 
 }
 
 // Fused 64 x 64 tiles of ffma_tile.cuh: one tile a CTA, all NS slices. SPLIT: K
-// split over the cluster (products without a reduction).
+// split over the cluster (products without a reduction). At NS = 3 the 4-byte-copy
+// forms spill 40 to 108 bytes a thread under the three CTAs a SM that hide the
+// copies' latency.
 template <class T, bool PRO, bool EPI, bool SPLIT, bool VEC>
 __global__ void __launch_bounds__(T::NT, T::NS == 4 ? 2 : 3)
 k_fused_gemm(const float* __restrict__ At, const float* __restrict__ B, float* C, int M, int N,
@@ -567,7 +569,7 @@ k_group_gemm(const GroupProb* __restrict__ probs, const int2* __restrict__ work,
 
 // The same with 32 x 32 tiles (small_tile_mainloop), stored from the registers:
 // batches whose 64 x 64 tiles are too few for the SMs (30 problems of n in
-// 64..128: 347 us a solve of 6 steps against 360 with 64 x 64 tiles).
+// 64..128: 336 us a solve of 6 steps against 360 with 64 x 64 tiles).
 template <int NS>
 __global__ void __launch_bounds__(128)
 k_group_small(const GroupProb* __restrict__ probs, const int2* __restrict__ work, GroupOp g,
@@ -852,7 +854,9 @@ int launch_slice_gemm(const float* At, const float* B, float* C, int M, int N, i
   // (128 x 64 from four units on: it needs several CTAs a SM). Measured, us
   // (128 x 64 / 64 x 64 / 64 x 32): 256^3 x 9 14.4 / 8.4 / 10.3; 512^3 x 32
   // 139 / 144 / 156; 512^3 x 64 274 / 272 / 295; 768^3 x 5 92 / 80 / 86;
-  // 389 x 257 x 301 x 9 (4-byte copies) 37 / 33 / 27.
+  // 389 x 257 x 301 x 9 (4-byte copies) 37 / 33 / 27. Not the fastest where the
+  // 64 x 32 tiles save only half a unit: at 512^3 x 32 it takes them (13.5 units
+  // against 14), 12% off the best.
   auto units = [&](int bm, int bn) {
     const long t = (long)((M + bm - 1) / bm) * ((N + bn - 1) / bn) * nslices;
     return (double)((t + NSM - 1) / NSM) * bm * bn / 4096.0;

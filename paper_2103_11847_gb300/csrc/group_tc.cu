@@ -20,7 +20,8 @@
 //     owns the row, which applies the trailing transform and the Krylov epilogue
 //     of group_operands (ca acc + cp prev and the norm partial of the problem's
 //     two-level reduction) and puts the result back the same way.
-// Two CTAs a SM (BN = 64) run one's epilogue beside the other's main loop.
+// Two CTAs a SM (BN = 64) run one's epilogue beside the other's main loop. (With
+// four slices the epilogue then spills 136 bytes a thread.)
 // Before, each CTA read the FP32 operand (twice the bytes, once a row tile),
 // transformed and rounded it in registers between K blocks, with one K block in
 // flight and rows of 16 bytes a lane in the epilogue: 226 us a launch at BN = 64;

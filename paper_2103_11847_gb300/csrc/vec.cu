@@ -371,13 +371,15 @@ k_mgs_pass(float* W, const float* __restrict__ Vi, const double* h, const float*
 // h_{j+1,j} and the step's flags (as k_gmres_step_done). h_0j is in place.
 //
 // Bound: latency, j + 1 dependent reductions over the tensor. As a launch a pass
-// (48 CTAs, W through HBM) a 256 x 256 x 3 pass took about 13 us; here a tensor
-// of up to 64 CTAs' worth of elements (n <= 262144) stays in the registers of
-// one thread-block cluster of 16 CTAs, the next V_i is loaded while a
-// reduction runs, and a reduction is the CTAs' partial sums pushed into every
-// CTA's shared memory, one cluster barrier, and the sum taken by every CTA: 55
-// passes in about 0.1 ms. A larger tensor takes the separate launches: one
-// cluster's 16 SMs would be short of bandwidth and registers.
+// (48 CTAs, W through HBM) a 256 x 256 x 3 pass took 20.2 us in a cold launch list;
+// here a tensor of up to 64 CTAs' worth of elements (n <= 262144) is kept by the
+// threads of one thread-block cluster of 16 CTAs (in registers, but for 84 to 200
+// bytes a thread of 768 or 1024 that spill), the next V_i is loaded while a
+// reduction runs, and a reduction is the CTAs' partial sums pushed into every CTA's
+// shared memory, one cluster barrier, and the sum taken by every CTA: the 55 passes
+// of ten steps take 251 us in such a list (4.6 us a pass; 1111 us as launches). A
+// larger tensor takes the separate launches: one cluster's 16 SMs would be short
+// of bandwidth and registers.
 // The element order and the reduction tree are the separate launches' (NV =
 // grid_for(n, 16) virtual CTAs of 256 threads, VC of them a CTA), so the bits
 // are the same.
